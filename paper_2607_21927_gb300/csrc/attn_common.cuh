@@ -51,7 +51,10 @@ __device__ __forceinline__ void key_range(const AttnArgs &a, const Task &t, int6
 __device__ __forceinline__ int64_t dense_suffix_start(const AttnArgs &a, int64_t i)
 {
     int64_t lo = i;
-    if (a.clique_B > 0) lo = min(lo, (i / a.clique_B) * a.clique_B);
+    if (a.clique_B > 0) {  // i and the block size are below 2^31
+        const uint32_t B = (uint32_t)a.clique_B;
+        lo = min(lo, (int64_t)((uint32_t)i / B * B));
+    }
     if (a.window > 1) lo = min(lo, max((int64_t)0, i - (int64_t)a.window + 1));
     return lo;
 }
