@@ -4,27 +4,29 @@
 //
 // Where the master mask keeps a large share of the causal pairs (union densities of tens of
 // percent, and the dense mode) a dense 128 x 128 score tile with the mask applied as -inf
-// beats gathering rows pair by pair. One CTA owns one (128-query tile, query head, set):
+// beats gathering rows pair by pair. One CTA owns one (128-query tile, query head, set). At head
+// dim 128 two CTAs form a cluster that shares its key and value tiles (two heads of a KV group, or
+// two query tiles where a group has an odd number of heads) and runs every product as one
+// 256-row product over both SMs (see Lay):
 //
-//   warp 8 (TMA)   streams 128-key tiles of the keys (64 KB: hi parts and corrections) and of
-//                  the values (fp16, 32 KB) in 128-byte swizzled boxes into two two-stage
-//                  shared-memory rings: a key stage is refilled as soon as its score products
-//                  are done, a value stage once its value product is; it also waits for each
-//                  tile's values to land and then arrives on that tile's P_FULL barrier, so
-//                  that the MMA warp waits once per value product;
-//   warp 9 (MMA)   issues tcgen05.mma: the score tile S (A = the query tile: its hi part in TMEM,
-//                  its low part in shared memory) into a double-buffered TMEM score tile, and
-//                  O += P V (A = P as fp16 in TMEM) into the TMEM output tile, committing each
-//                  step to an mbarrier; TMEM holds S twice (2 x 128 columns), O (128), the
-//                  query's hi part (64) and P (64), all 512 columns. P has columns of its own, so
-//                  the scores of tile j + 2 start as soon as those of tile j have been read;
-//   warps 0-7      two groups of four warps, one thread per query row in each, taking alternate
-//                  tiles: write the query tile, then per tile tcgen05.ld the row's 128 scores,
-//                  apply the bitmap (words fetched four tiles ahead) or the causal cut, take the
-//                  row max, pass the row's reference maximum on to the other group, fp32 online
-//                  softmax with lazy rescaling of O in TMEM (only when the row max grows by more
-//                  than 2^8), write P into TMEM, and at the end normalise O (and undo the values'
-//                  power-of-two scale) and store the row.
+//   warp 8 (TMA)    loads the query tile, then streams 128-key tiles of the keys (hi parts and
+//                   corrections) and of the values (fp16) in 128-byte swizzled boxes into two
+//                   shared-memory rings, each CTA its half: a key stage is refilled as soon as its
+//                   score products are done, a value stage once its value product is;
+//   warp 11 (relay) passes what has landed in either CTA on to the barriers of the issuing warps;
+//   warps 9, 10     (of the cluster's first CTA) issue tcgen05.mma: warp 9 the score tile S (query
+//                   and keys from shared memory) into a double-buffered TMEM score tile, warp 10
+//                   O += P V (A = P as fp16 in TMEM, double-buffered) into the TMEM output tile,
+//                   committing each step to an mbarrier of both CTAs. TMEM holds S (2 x 128
+//                   columns), O (128) and P (2 x 64), all 512 columns. P has columns of its own,
+//                   so the scores of tile j + 2 start as soon as those of tile j have been read;
+//   warps 0-7       two groups of four warps, one thread per query row in each, taking alternate
+//                   tiles: per tile tcgen05.ld the row's 128 scores, apply the bitmap (words
+//                   fetched four tiles ahead) or the causal cut, take the row max, fp32 online
+//                   softmax from the reference maximum that the other group hands over, with lazy
+//                   rescaling of O in TMEM (only when the row max grows by more than 2^14), write P
+//                   into TMEM, and at the end normalise O (and undo the values' power-of-two
+//                   scale) and store it, coalesced, through shared memory.
 //
 // Precision. With activation outlier channels the scores reach tens of units while the
 // output moves by p (v_j - o) per unit of score error, so the scores need about 17
@@ -49,12 +51,22 @@
 //                         operand moves, as long as the product, plus its waits;
 //   2,055 / 2,400         operands warp-uniform and issued by an elected lane: the softmax, its two
 //                         threads per row meeting in every tile, set the pace;
-//   1,860 / 2,040         the two groups on alternate tiles, half a period apart (this form): the
-//                         rest is the L2 latency of the keys, requested only when the ring's
-//                         two stages allow, and the issuer's waits.
-// Layer calls, before -> now: N = 8192 305 -> 279 us, 32k dense 3.73 -> 3.32 ms, 64k 14.0 -> 12.6 ms.
-// A separate issuing warp for the value products ran no faster (its products interleave with the
-// next scores, whose keys then arrive later still).
+//   1,860 / 2,040         the two groups on alternate tiles, half a period apart; a separate warp
+//                         for the value products then made it 2,030 / 2,170: 96 KB of keys and
+//                         values per tile and SM (17 TB/s at this pace) came in too late;
+//   1,720 / 1,985         tiles shared by two SMs;
+//   1,620 / 1,950         P double-buffered: dense, the tensor pipe is 95% busy and the power limit
+//                         holds the clock at 1.58 GHz; with a bitmap the softmax (about 450 cycles of
+//                         masking per tile more) is as slow as the pipe. There the groups' warps of a
+//                         scheduler ran their exponentials against each other, and a warp in a
+//                         hundred rescaled O, while seven others waited: the reference maximum is now
+//                         handed over after the exponentials, and moves at 2^14 instead of 2^8.
+// A CTA's start and end, 16,000 cycles with the query rows loaded and the output rows stored 16 bytes
+// per lane and row, take 7,000 with the query tile loaded by TMA and the output through
+// shared memory.
+// Layer calls, before -> now: N = 8192 306 -> 248 us, 32k dense 3.77 -> 2.98 ms, 64k 14.1 -> 11.5 ms.
+// Not kept: more polls between two reads of the error word in a wait (3% slower at N = 8192), a
+// suspend-time hint on the polls (no change).
 //
 // The suffix pass of the dense-suffix split (SUFFIX) runs the same pipeline over the key
 // tiles of each row's dense suffix only (its Structural block and / or local window: every key
@@ -91,46 +103,72 @@ constexpr int BN = 128;          // keys per stage
 // scores of a tile stay in registers.
 constexpr int kGroupWarps = 4;
 constexpr int kSoftmaxWarps = 2 * kGroupWarps;
-constexpr int kSoftmaxThreads = 32 * kSoftmaxWarps;
-constexpr int kTmaWarp = kSoftmaxWarps, kMmaWarp = kSoftmaxWarps + 1;
+constexpr int kTmaWarp = kSoftmaxWarps, kScoreWarp = kSoftmaxWarps + 1, kValueWarp = kSoftmaxWarps + 2,
+              kRelayWarp = kSoftmaxWarps + 3;
 constexpr int kThreads = 32 * (kSoftmaxWarps + 4);
 // registers per thread: at launch, then after setmaxnreg of a softmax and of a loader / MMA thread
 constexpr int kRegs = 168, kSoftmaxRegs = 200, kOtherRegs = 104;
 static_assert(2 * kSoftmaxRegs + kOtherRegs == 3 * kRegs, "the shares of the three warpgroups add up to the launch's");
-constexpr uint32_t kTmemCols = 512;  // S[2] (2 x 128) + O (128) + Q hi (64) + P (64)
+// The reference maximum of a row moves only when its maximum grows by more than this (log2): P
+// stays below 2^14, inside fp16, and a lower reference only keeps more of the small weights out of
+// fp16's subnormals. On a 10% mask of 64k tokens one warp in a hundred rescaled O in a tile at a
+// step of 2^8, and a tile waits for the slowest of eight warps.
+constexpr float kLazyLog2 = 14.f;
+constexpr uint32_t kTmemCols = 512;  // S (2 x 128) + O (128) + P (2 x 64)
 
-// shared-memory map (bytes, from a 1024-aligned base) for head dim DT (128 or 64): the K ring,
-// the V ring, the low part of the query tile, then the barriers, the TMEM base and what the two
-// threads of a row hand to each other: the row's reference maximum after each tile, and at the
-// end each thread's row sum and the maximum it refers to
-constexpr int KV_BLK = BN * 128;            // 16 KB: one 64-column block
-constexpr int kStages = 2;                  // stages of each ring
+// How the kernel of head dim DT (128 or 64) is laid out. At 128 two CTAs of a cluster share their
+// key and value tiles (CG = 2: tcgen05 cta_group::2, one 256 x 128 product over both SMs, each
+// holding half of the B operand: 64 of a tile's keys, 64 of the head dim's value columns). That
+// halves the L2 traffic of the tiles (96 KB per tile and SM would be near the L2's whole
+// bandwidth at the tensor pipe's rate) and leaves shared memory for a key ring of four stages, past
+// the latency of a load, beside the query tile. At 64 the halves of the value columns would be
+// 64-byte rows; each CTA works for itself there.
+//
+// Shared memory (bytes, from a 1024-aligned base): the K ring, the V ring, the query tile (hi part,
+// low part), then the barriers, the TMEM base and what the two threads of a row hand to each
+// other: the row's reference maximum after each tile, and at the end each thread's row sum and
+// the maximum it refers to.
 template <int DT>
-struct Smem {
-    static constexpr int KV_ARR = BN * DT * 2;  // 32 KB at DT = 128: one of K hi / K lo / V / Q lo
-    static constexpr int K_STAGE = 2 * KV_ARR;  // K hi, K lo
-    static constexpr int V_STAGE = KV_ARR;
+struct Lay {
+    static constexpr int CG = DT == 128 ? 2 : 1;
+    static constexpr int NSK = 4, NSV = 2;       // stages of the key and of the value ring
+    static constexpr int NB = DT / 64;           // 64-column blocks of a row
+    static constexpr int KROWS = BN / CG;        // keys of a tile held by one CTA
+    static constexpr int K_BLK = KROWS * 128;    // one 64-column block of K hi or K lo
+    static constexpr int K_ARR = NB * K_BLK;     // K hi or K lo
+    static constexpr int K_STAGE = 2 * K_ARR;
+    static constexpr int V_BLK = BN * 128;
+    static constexpr int V_STAGE = NB / CG * V_BLK;
+    static constexpr int Q_BLK = BM * 128;
     static constexpr int OFF_K = 0;
-    static constexpr int OFF_V = kStages * K_STAGE;
-    static constexpr int OFF_Q = OFF_V + kStages * V_STAGE;
-    static constexpr int OFF_BARS = OFF_Q + KV_ARR;
-    static constexpr int OFF_TMEM = OFF_BARS + 120;  // after the NBAR barriers
-    static constexpr int OFF_M = OFF_BARS + 128;     // float [BM]
+    static constexpr int Q_ARR = NB * Q_BLK;     // Q hi or Q lo
+    static constexpr int OFF_V = NSK * K_STAGE;
+    static constexpr int OFF_Q = OFF_V + NSV * V_STAGE;
+    static constexpr int OFF_BARS = OFF_Q + 2 * Q_ARR;
+    static constexpr int OFF_TMEM = OFF_BARS + 248;  // after the barriers
+    static constexpr int OFF_M = OFF_BARS + 256;     // float [BM]
     static constexpr int OFF_ML = OFF_M + BM * 4;    // float2 [2][BM]
     static constexpr int BYTES = OFF_ML + 2 * BM * 8;
     static_assert(BYTES <= 232448, "shared memory of a CTA");
+    // Barriers, one of each kind per ring stage (a tile's stage is its number mod NSK or NSV), so
+    // that no waiter can fall two phases behind a barrier it polls by parity:
+    //   Q_FULL          the CTA's query tile has landed (relayed with the first keys)
+    //   K_FULL, V_FULL  the CTA's part of the tile's keys / values has landed (relayed to S_GO / P_GO)
+    //   S_GO            the score products of a tile may start: its keys have landed and the scores
+    //                   of the tile two before (if any) have been read out of their buffer
+    //   S_FULL          they are done (and the key stage is free)
+    //   P_GO            the value product may start: P is written and the values have landed
+    //   PV_DONE         it is done (P's buffer and the value stage are free, O has settled)
+    // S_GO and P_GO are those of the cluster's first CTA, whose warps issue the products; both CTAs
+    // arrive on them, and the products' completion arrives on S_FULL and PV_DONE of both.
+    static constexpr int B_Q_FULL = 0, B_K_FULL = 1, B_S_GO = B_K_FULL + NSK, B_S_FULL = B_S_GO + NSK,
+                         B_V_FULL = B_S_FULL + NSK, B_P_GO = B_V_FULL + NSV, B_PV_DONE = B_P_GO + NSV,
+                         B_END = B_PV_DONE + NSV, NBAR = B_END + 2;
+    static_assert(NBAR * 8 <= 248, "barriers below the TMEM base word");
 };
-// the head-dim-128 layout (232,064 of the 232,448 bytes a CTA can have) is requested at either
+// the head-dim-128 layout (232,192 of the 232,448 bytes a CTA can have) is requested at either
 // head dim: it keeps one CTA per SM, as the CTA holds all 512 TMEM columns
-constexpr int SMEM_BYTES = Smem<128>::BYTES;
-
-// S_FULL, S_READ, P_FULL and PV_DONE have one barrier per tile parity, so that no waiter can
-// fall two phases behind a barrier it polls by parity.
-enum Bar {
-    B_Q = 0, B_K_FULL = 1, B_V_FULL = 3, B_S_FULL = 5, B_S_READ = 7, B_P_FULL = 9, B_PV_DONE = 11, B_END = 13,
-    NBAR = 14
-};
-static_assert(NBAR * 8 <= 120, "barriers below the TMEM base word");
+constexpr int SMEM_BYTES = Lay<128>::BYTES;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -141,6 +179,26 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// Arrival on a barrier of any CTA of the cluster (shared::cluster address, see cluster_addr). What
+// it announces is tensor memory that was read or written (ordered by tcgen05.wait and
+// tcgen05.fence) or a copy that landed, not this thread's memory accesses: releasing those at
+// cluster scope took 1,000 cycles and more per arrival (a tile of a 32k dense layer took
+// 3,130 cycles instead of 1,720).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
+{
+    uint32_t d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+    return d;
+}
+// All threads of the cluster's CTAs.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
 {
@@ -239,8 +297,10 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool b_mn_major)
 }
 
 // A operand from TMEM (rows in lanes, 16-bit values packed two per column), B from shared memory.
+template <int CG>
 __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b, uint32_t idesc, uint32_t acc)
 {
+    if constexpr (CG == 1)
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
         "mov.b64 db, {%2, %5};\n\t"
@@ -248,12 +308,22 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a_tmem), "r"(b), "r"(idesc), "r"(acc), "n"(kDescHi)
         : "memory");
+    else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "r"(b), "r"(idesc), "r"(acc), "n"(kDescHi)
+        : "memory");
 }
 
 // kind::f8f6f4 (e4m3 x e4m3 with the instruction descriptor's format fields 0), A and B from
 // shared memory.
+template <int CG>
 __device__ __forceinline__ void tc_mma_ss_f8(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t acc)
 {
+    if constexpr (CG == 1)
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
         "mov.b64 da, {%1, %5};\n\t"
@@ -262,11 +332,22 @@ __device__ __forceinline__ void tc_mma_ss_f8(uint32_t d_tmem, uint32_t a, uint32
         "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a), "r"(b), "r"(idesc), "r"(acc), "n"(kDescHi)
         : "memory");
+    else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %5};\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(idesc), "r"(acc), "n"(kDescHi)
+        : "memory");
 }
 
 // A and B from shared memory, 16-bit values.
+template <int CG>
 __device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, uint32_t acc)
 {
+    if constexpr (CG == 1)
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
         "mov.b64 da, {%1, %5};\n\t"
@@ -275,23 +356,70 @@ __device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint32_t a, uint32_t 
         "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a), "r"(b), "r"(idesc), "r"(acc), "n"(kDescHi)
         : "memory");
-}
-
-// kind::f16 accumulating onto D scaled by 2^-12 on entry: D = A B + 2^-12 D.
-__device__ __forceinline__ void tc_mma_ts_scaled12(uint32_t d_tmem, uint32_t a_tmem, uint32_t b, uint32_t idesc)
-{
+    else
     asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %5};\n\t"
         "mov.b64 db, {%2, %5};\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p, 12;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "r"(b), "r"(idesc), "r"(1u), "n"(kDescHi)
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(idesc), "r"(acc), "n"(kDescHi)
         : "memory");
 }
 
+// kind::f16 accumulating onto D scaled by 2^-12 on entry: D = A B + 2^-12 D.
+template <int CG>
+__device__ __forceinline__ void tc_mma_ss_scaled12(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc)
+{
+    if constexpr (CG == 1)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %5};\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p, 12;\n\t}" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(idesc), "r"(1u), "n"(kDescHi)
+        : "memory");
+    else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %5};\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p, 12;\n\t}" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(idesc), "r"(1u), "n"(kDescHi)
+        : "memory");
+}
+
+// Arrive on the barrier (CG = 2: of both CTAs) once this thread's products so far are done.
+template <int CG>
 __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    if constexpr (CG == 1)
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+                     "h"((uint16_t)3)
+                     : "memory");
+}
+template <int CG>
+__device__ __forceinline__ void tmem_alloc(uint32_t dst)
+{
+    if constexpr (CG == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    } else {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+}
+template <int CG>
+__device__ __forceinline__ void tmem_dealloc(uint32_t tmem)
+{
+    if constexpr (CG == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp gets lane (base + t).
@@ -333,17 +461,6 @@ __device__ __forceinline__ void pin64(uint32_t *v)
                      "+r"(v[i + 6]), "+r"(v[i + 7]));
 }
 
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t *v)
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
-        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-        : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
 // 32 columns, not waited for (tmem_wait_st).
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t *v)
 {
@@ -353,21 +470,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t *v)
         : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// 32 lanes x 16 consecutive 32-bit columns, loaded and waited for in one statement.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // max of three floats in one instruction
 __device__ __forceinline__ float fmax3(float x, float y, float z)
@@ -443,16 +545,16 @@ __device__ __forceinline__ int64_t row_word_offset(int64_t i)
     return i + 16 * a * (a - 1) + a * b;
 }
 
+// 16 bytes of outputs (four fp32 or eight bf16 values)
 template <typename TOut>
-__device__ __forceinline__ void store8(TOut *dst, const float *x);
+__device__ __forceinline__ void store16(void *dst, const float *x);
 template <>
-__device__ __forceinline__ void store8<float>(float *dst, const float *x)
+__device__ __forceinline__ void store16<float>(void *dst, const float *x)
 {
-    reinterpret_cast<float4 *>(dst)[0] = make_float4(x[0], x[1], x[2], x[3]);
-    reinterpret_cast<float4 *>(dst)[1] = make_float4(x[4], x[5], x[6], x[7]);
+    *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
 }
 template <>
-__device__ __forceinline__ void store8<__nv_bfloat16>(__nv_bfloat16 *dst, const float *x)
+__device__ __forceinline__ void store16<__nv_bfloat16>(void *dst, const float *x)
 {
     uint4 w;
     w.x = pack_bf16(x[0], x[1]);
@@ -463,218 +565,226 @@ __device__ __forceinline__ void store8<__nv_bfloat16>(__nv_bfloat16 *dst, const 
 }
 
 struct TileMaps {
-    CUtensorMap kh, kl, v;
+    CUtensorMap qh, ql, kh, kl, v;
 };
 
 template <int DT, bool SPLIT, bool DENSE, bool SUFFIX, typename TOut>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_attn_tile(const AttnArgs a, const __grid_constant__ TileMaps maps, const void *q_hi, const void *q_lo)
+    k_attn_tile(const AttnArgs a, const __grid_constant__ TileMaps maps)
 {
     static_assert(DT == 128 || DT == 64, "head dim 64 or 128");
-    constexpr int KV_ARR = Smem<DT>::KV_ARR, K_STAGE = Smem<DT>::K_STAGE, V_STAGE = Smem<DT>::V_STAGE;
-    constexpr int OFF_K = Smem<DT>::OFF_K, OFF_V = Smem<DT>::OFF_V, OFF_Q = Smem<DT>::OFF_Q;
-    constexpr int NB = DT / 64;  // 64-column blocks of a row
+    using L = Lay<DT>;
+    constexpr int CG = L::CG, NSK = L::NSK, NSV = L::NSV, NB = L::NB;
     // no static shared memory: the dynamic block starts where the CTA's window does
     extern __shared__ __align__(1024) unsigned char smem[];
-    uint64_t *const bars = reinterpret_cast<uint64_t *>(smem + Smem<DT>::OFF_BARS);
-    uint32_t &tmem_base_sh = *reinterpret_cast<uint32_t *>(smem + Smem<DT>::OFF_TMEM);
-    float *const m_sh = reinterpret_cast<float *>(smem + Smem<DT>::OFF_M);
-    float2(*const ml_sh)[BM] = reinterpret_cast<float2(*)[BM]>(smem + Smem<DT>::OFF_ML);
+    uint64_t *const bars = reinterpret_cast<uint64_t *>(smem + L::OFF_BARS);
+    uint32_t &tmem_base_sh = *reinterpret_cast<uint32_t *>(smem + L::OFF_TMEM);
+    float *const m_sh = reinterpret_cast<float *>(smem + L::OFF_M);
+    float2(*const ml_sh)[BM] = reinterpret_cast<float2(*)[BM]>(smem + L::OFF_ML);
     const uint32_t sbase = smem_u32(smem);
-    if ((sbase & 1023u) != 0u) {  // the swizzled boxes need it; the same for every thread
-        if (threadIdx.x == 0) atomicOr(&g_ris_tile_error, 2u);
-        return;
-    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    // ---- tile of this CTA (tiles covering rows row0 .. row1-1): heavier (later) tiles first
-    const int qt_end = (int)((a.row1 + BM - 1) / BM);
-    const int64_t b = blockIdx.x;
-    const int h = (int)(b % a.Hq);
-    const int64_t r2 = b / a.Hq;
-    const int s = (int)(r2 % a.n_sets);
-    const int qt = qt_end - 1 - (int)(r2 / a.n_sets);
-    const int64_t q0 = (int64_t)qt * BM;
+    // ---- tile of this CTA (tiles covering rows row0 .. row1-1): heavier (later) tiles first. The
+    // two CTAs of a cluster take two heads of a KV group at the same query tile or, where a group
+    // has an odd number of heads, two consecutive query tiles of a head; either way the same key
+    // tiles. A query tile outside the row range (the second of an odd last one) has no rows.
+    const int qt_end = (int)((a.row1 + BM - 1) / BM), qt_first = (int)(a.row0 / BM);
+    const int rank = CG == 2 ? (int)(blockIdx.x & 1) : 0;
+    const bool head_pair = CG == 2 && (a.G & 1) == 0;
+    const unsigned n_h = (unsigned)(head_pair ? a.Hq / 2 : a.Hq);
+    const unsigned b = blockIdx.x / CG, r2 = b / n_h;
+    const int h = head_pair ? 2 * (int)(b - r2 * n_h) + rank : (int)(b - r2 * n_h);
+    const int s = (int)(r2 % (unsigned)a.n_sets), qp = (int)(r2 / (unsigned)a.n_sets);
+    const int qt_hi = CG == 2 && !head_pair ? qt_end - 1 - 2 * qp : qt_end - 1 - qp;
+    const int qt_lo = CG == 2 && !head_pair ? qt_hi - 1 : qt_hi;
+    const int64_t q0 = (int64_t)(rank == 0 ? qt_hi : CG == 2 && !head_pair ? qt_lo : qt_hi) * BM;
     const int g = h / a.G;
     const int mask_id = s * a.heads_keyed + (a.heads_keyed > 1 ? g : 0);
-    const int64_t last_row = (q0 + BM - 1 < a.row1 - 1) ? q0 + BM - 1 : a.row1 - 1;
+    const int64_t last_row = min((int64_t)qt_hi * BM + BM - 1, a.row1 - 1);
     // causal: key tiles kt0 .. last_row / BN (kt0 = 0, or the tile of the first row's dense
-    // suffix start, the earliest of the tile's rows)
-    const int kt0 = SUFFIX ? (int)(dense_suffix_start(a, q0) / BN) : 0;
+    // suffix start, the earliest of the cluster's rows)
+    const int kt0 = SUFFIX ? (int)(dense_suffix_start(a, (int64_t)max(qt_lo, qt_first) * BM) / BN) : 0;
     const int n_kt = (int)(last_row / BN) + 1 - kt0;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < NBAR; ++i) {
+        for (int i = 0; i < L::NBAR; ++i) {
             uint32_t cnt = 1;
-            if (i == B_Q) cnt = kSoftmaxThreads;
-            if (i == B_S_READ || i == B_S_READ + 1) cnt = kGroupWarps;
-            if (i == B_P_FULL || i == B_P_FULL + 1) cnt = kGroupWarps + 1;  // + the loader's relay
+            // the group's warps and the relay, of each CTA
+            if ((i >= L::B_S_GO && i < L::B_S_GO + NSK) || (i >= L::B_P_GO && i < L::B_P_GO + NSV)) cnt = (kGroupWarps + 1) * CG;
             mbar_init(smem_u32(&bars[i]), cnt);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == kMmaWarp) {  // TMEM allocation by one full warp
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)),
-                     "r"(kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == kScoreWarp) tmem_alloc<CG>(smem_u32(&tmem_base_sh));  // by one full warp (of each CTA)
+    __syncwarp();
     tc_fence_before();
+    if constexpr (CG == 2) cluster_sync();
     __syncthreads();
     tc_fence_after();
     // all 512 columns: the allocation starts at TMEM address 0, so every address below is a
     // constant (anything else ends the CTA as a failed wait does, below)
-    constexpr uint32_t T_S0 = 0, T_O = T_S0 + 2 * BN, T_Q = T_O + DT, T_P = T_Q + DT / 2;
-    static_assert(T_P + BN / 2 <= kTmemCols, "TMEM columns");
+    constexpr uint32_t T_S0 = 0, T_O = T_S0 + 2 * BN, T_P0 = T_O + DT;
+    static_assert(T_P0 + BN <= kTmemCols, "TMEM columns");
     const uint32_t tmem = tmem_base_sh;
-    constexpr auto BAR = [](int i) { return (uint32_t)(Smem<DT>::OFF_BARS + 8 * i); };
+    constexpr auto BAR = [](int i) { return (uint32_t)(L::OFF_BARS + 8 * i); };
+    const uint32_t lead = CG == 2 ? cluster_addr(sbase, 0) : sbase;  // the issuing CTA's shared memory
+    auto arrive_lead = [&](int bar) {
+        if constexpr (CG == 2)
+            mbar_arrive_cluster(lead + BAR(bar));
+        else
+            mbar_arrive(sbase + BAR(bar));
+    };
     const long long wl = a.wait_limit > 0 ? (long long)a.wait_limit : (1LL << 31);
-    bool ok = tmem == 0u;
+    bool ok = tmem == 0u && (sbase & 1023u) == 0u;  // (the swizzled boxes need the alignment)
 
     if (warp >= kSoftmaxWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
     if (!ok) {
-        // unexpected TMEM base: straight to the common end
+        // an unexpected base: straight to the common end
     } else if (warp == kTmaWarp) {
         // =============================== TMA producer
         if (lane == 0 && a.debug_no_loads == 0) {
-            // Keys of tile j once the score products of tile j - 2 are done, values of tile j once the
-            // value product of tile j - 2 is. The ring stages and the score buffers are both
-            // indexed by tile parity, so the loader waits on the barriers that announce those
-            // products (S_FULL, PV_DONE) instead of on barriers of its own, which saves the tensor
-            // pipe two commits per tile. The keys are requested ahead of the values: the score
-            // products of tile t + 1 finish before the value product of tile t - 2, so in this
-            // order no wait holds up a load that could go before it.
-            // The loader also waits for each tile's values to land and then arrives on that tile's
-            // P_FULL (which counts the softmax warps and this one), so that the MMA warp waits
-            // once before a value product instead of twice.
-            static_assert(kStages == 2, "ring stages share the parity of the score buffers");
-            int nk = 0, nv = 0, nr = 0;  // tiles whose keys / values were requested; values relayed
-            auto load_k = [&](int j) {
-                const uint32_t bk = smem_u32(&bars[B_K_FULL + j % kStages]);
-                const uint32_t dk = sbase + OFF_K + (j % kStages) * K_STAGE;
-                mbar_arrive_expect_tx(bk, (SPLIT ? 2 : 1) * KV_ARR);
+            // The query tile and the first keys, then keys of tile j once the score products of tile
+            // j - NSK are done, values of tile j once the value product of tile j - NSV is: the loader
+            // waits on the barriers that announce those products (S_FULL, PV_DONE) instead of on
+            // barriers of its own, which saves the tensor pipe two commits per tile. The score
+            // products of tile t + 1 finish before the value product of tile t, so in this order no
+            // wait holds up a load that could go before it.
+            int nk = 0, nv = 0;  // tiles whose keys / values were requested
+            auto load_k = [&](int j) -> bool {
+                if (j >= n_kt) return true;
+                const int st = j % NSK;
+                if (j >= NSK && !mbar_wait(sbase + BAR(L::B_S_FULL + st), (j / NSK - 1) & 1, wl)) return false;
+                const uint32_t bk = sbase + BAR(L::B_K_FULL + st);
+                const uint32_t dk = sbase + L::OFF_K + st * L::K_STAGE;
+                const int key = (kt0 + j) * BN + L::KROWS * rank;
+                mbar_arrive_expect_tx(bk, (SPLIT ? 2 : 1) * L::K_ARR);
                 for (int blk = 0; blk < NB; ++blk) {
-                    tma_load_3d(dk + blk * KV_BLK, &maps.kh, 64 * blk, g, (kt0 + j) * BN, bk);
-                    if (SPLIT) tma_load_3d(dk + KV_ARR + blk * KV_BLK, &maps.kl, 64 * blk, g, (kt0 + j) * BN, bk);
+                    tma_load_3d(dk + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
+                    if (SPLIT) tma_load_3d(dk + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
                 }
                 nk = j + 1;
-            };
-            auto load_v = [&](int j) {
-                const uint32_t bv = smem_u32(&bars[B_V_FULL + j % kStages]);
-                const uint32_t dv = sbase + OFF_V + (j % kStages) * V_STAGE;
-                mbar_arrive_expect_tx(bv, KV_ARR);
-                for (int blk = 0; blk < NB; ++blk) tma_load_3d(dv + blk * KV_BLK, &maps.v, 64 * blk, g, (kt0 + j) * BN, bv);
-                nv = j + 1;
-            };
-            auto relay = [&](int jv) -> bool {
-                if (!mbar_wait(smem_u32(&bars[B_V_FULL + jv % kStages]), (jv / kStages) & 1, wl)) return false;
-                mbar_arrive(smem_u32(&bars[B_P_FULL + (jv & 1)]));
-                nr = jv + 1;
                 return true;
             };
-            for (int j = 0; j < kStages && j < n_kt; ++j) {
-                load_k(j);
-                load_v(j);
-            }
-            auto next_k = [&](int j) -> bool {  // into the stage that tile j - 2 leaves
+            auto load_v = [&](int j) -> bool {
                 if (j >= n_kt) return true;
-                if (!mbar_wait(smem_u32(&bars[B_S_FULL + (j & 1)]), ((j - kStages) >> 1) & 1, wl)) return false;
-                load_k(j);
+                const int st = j % NSV;
+                if (j >= NSV && !mbar_wait(sbase + BAR(L::B_PV_DONE + st), (j / NSV - 1) & 1, wl)) return false;
+                const uint32_t bv = sbase + BAR(L::B_V_FULL + st);
+                const uint32_t dv = sbase + L::OFF_V + st * L::V_STAGE;
+                mbar_arrive_expect_tx(bv, L::V_STAGE);
+                for (int blk = 0; blk < NB / CG; ++blk)
+                    tma_load_3d(dv + blk * L::V_BLK, &maps.v, 64 * (blk + rank), g, (kt0 + j) * BN, bv);
+                nv = j + 1;
                 return true;
             };
-            ok = next_k(kStages);
-            for (int t = 0; t < n_kt && ok; ++t) {
-                ok = next_k(t + kStages + 1);
-                if (ok && t >= 1) ok = relay(t - 1);
-                if (!ok) break;
-                if (t >= kStages) {
-                    ok = mbar_wait(smem_u32(&bars[B_PV_DONE + (t & 1)]), ((t - kStages) >> 1) & 1, wl);
-                    if (!ok) break;
-                    load_v(t);
-                }
+            const uint32_t bq = sbase + BAR(L::B_Q_FULL);
+            mbar_arrive_expect_tx(bq, (SPLIT ? 2 : 1) * L::Q_ARR);
+            for (int blk = 0; blk < NB; ++blk) {  // rows outside the tensor read as zeros
+                tma_load_3d(sbase + L::OFF_Q + blk * L::Q_BLK, &maps.qh, 64 * blk, h, (int)(q0 - a.q_first), bq);
+                if (SPLIT) tma_load_3d(sbase + L::OFF_Q + L::Q_ARR + blk * L::Q_BLK, &maps.ql, 64 * blk, h, (int)(q0 - a.q_first), bq);
             }
-            if (ok && nr < n_kt) ok = relay(n_kt - 1);
+            ok = load_k(0) && load_v(0) && load_k(1) && load_v(1) && load_k(2) && load_k(3) && load_k(4);
+            for (int t = 0; t < n_kt && ok; ++t) ok = load_k(t + 5) && load_v(t + 2);
             // let the copies requested last into each stage land before the CTA can leave
             // (earlier ones were consumed before their stage was refilled)
-            for (int j = nk - kStages; j < nk; ++j)
-                if (j >= 0) mbar_wait_own(smem_u32(&bars[B_K_FULL + j % kStages]), (j / kStages) & 1);
-            for (int j = nv - kStages; j < nv; ++j)
-                if (j >= 0) mbar_wait_own(smem_u32(&bars[B_V_FULL + j % kStages]), (j / kStages) & 1);
+            mbar_wait_own(bq, 0);
+            for (int j = nk - NSK; j < nk; ++j)
+                if (j >= 0) mbar_wait_own(sbase + BAR(L::B_K_FULL + j % NSK), (j / NSK) & 1);
+            for (int j = nv - NSV; j < nv; ++j)
+                if (j >= 0) mbar_wait_own(sbase + BAR(L::B_V_FULL + j % NSV), (j / NSV) & 1);
+            static_assert(NSK == 4 && NSV == 2, "the order of the loads and of the relay");
         }
-    } else if (warp == kMmaWarp) {
-        // =============================== MMA issuer
+    } else if (warp == kRelayWarp) {
+        // =============================== relay: what has landed, to the barriers that the issuing
+        // warps wait on, in the order of the loads; so each of them waits on one barrier per tile
+        if (lane == 0) {
+            auto relay_k = [&](int j) -> bool {
+                if (j >= n_kt) return true;
+                if (!mbar_wait(sbase + BAR(L::B_K_FULL + j % NSK), (j / NSK) & 1, wl)) return false;
+                arrive_lead(L::B_S_GO + j % NSK);
+                return true;
+            };
+            auto relay_v = [&](int j) -> bool {
+                if (j >= n_kt) return true;
+                if (!mbar_wait(sbase + BAR(L::B_V_FULL + j % NSV), (j / NSV) & 1, wl)) return false;
+                arrive_lead(L::B_P_GO + j % NSV);
+                return true;
+            };
+            ok = mbar_wait(sbase + BAR(L::B_Q_FULL), 0, wl) && relay_k(0) && relay_v(0) && relay_k(1) && relay_v(1) &&
+                 relay_k(2) && relay_k(3) && relay_k(4);
+            for (int t = 0; t < n_kt && ok; ++t) ok = relay_k(t + 5) && relay_v(t + 2);
+        }
+    } else if (rank == 0) {
+        // =============================== product issuers (of the cluster's first CTA, for both): one
+        // warp for the scores, one for the value products, so that neither's waits (about 100
+        // cycles each even on a completed phase) leave the tensor pipe without queued work.
         // The whole warp runs this code, so that every operand is warp-uniform, and one elected
         // lane issues: inside a branch on the lane the compiler moves each of a product's operands
         // (two descriptors, two TMEM addresses, the instruction descriptor) into uniform registers
         // one by one, about 60 cycles per product, as long as a 128 x 128 x 16 product itself.
-        constexpr uint32_t ID_S = idesc_bf16(BM, BN, false);  // S[128 x 128] = Q K^T, both K-major
-        constexpr uint32_t ID_SH = idesc_f16(BM, BN, false);  // fp16 x fp16 (and e4m3 x e4m3 for kind::f8f6f4)
-        constexpr uint32_t ID_O = idesc_f16(BM, DT, true);    // O[128 x DT] += P V, fp16, V MN-major
+        constexpr uint32_t ID_S = idesc_bf16(CG * BM, BN, false);  // S[128 x 128] = Q K^T, both K-major
+        constexpr uint32_t ID_SH = idesc_f16(CG * BM, BN, false);  // fp16 x fp16 (and e4m3 x e4m3 for kind::f8f6f4)
+        constexpr uint32_t ID_O = idesc_f16(CG * BM, DT, true);  // O[128 x DT] += P V, fp16, V MN-major
         // fp8-correction scores (rotated q / k at head dim 128, operands written by
         // launch_fp8_prep when the bounds allow): the same bytes in the same places as the
-        // bf16 pair, read as fp16 hi parts (query in TMEM, key bytes 0-255 of a row) and e4m3
-        // corrections (the 64-column blocks of the query's low part in shared memory and of
-        // the key's at KV_ARR: hi parts, then lo parts)
+        // bf16 pair, read as fp16 hi parts and, in the place of the low parts (Q_ARR, K_ARR on),
+        // e4m3 corrections, one 64-column block of hi parts and one of lo parts
         int ea = 0, eb = 0;
         const bool use8 = DT == 128 && SPLIT && a.qk_bound != nullptr &&
                           __any_sync(0xFFFFFFFFu, fp8_score_scales(a.qk_bound[0], a.qk_bound[1], ea, eb));
-        // score products of a tile whose parity (ring stage and score buffer) is ST
+        // score products of a tile of ring stage ST: A = the query tile, B = the keys, both K-major in
+        // shared memory, a k-step of 16 (e4m3: 32) columns 32 B further in a 128 B row
         auto issue_s = [&](auto st_c) {
             constexpr int ST = decltype(st_c)::value;
-            const uint32_t kd = desc_lo(sbase + OFF_K + ST * K_STAGE, 16);  // K hi; K lo KV_ARR on
-            const uint32_t qd = desc_lo(sbase + OFF_Q, 16);                  // Q lo
-            constexpr uint32_t dt = T_S0 + ST * BN;
+            const uint32_t kd = desc_lo(sbase + L::OFF_K + ST * L::K_STAGE, 16);  // K hi; K lo K_ARR on
+            const uint32_t qd = desc_lo(sbase + L::OFF_Q, 16);                     // Q hi; Q lo Q_ARR on
+            constexpr uint32_t dt = T_S0 + (ST & 1) * BN;
             if (elect_one()) {
                 if (use8) {
                     // 2^12 (q_h8 k_l8 + q_l8 k_h8): two e4m3 products of 4 k-steps of 32
 #pragma unroll
                     for (int ks = 0; ks < DT / 32; ++ks)
-                        tc_mma_ss_f8(dt, qd + dstep(ks * 32), kd + dstep(KV_ARR + KV_BLK + ks * 32), ID_SH, ks > 0);
+                        tc_mma_ss_f8<CG>(dt, qd + dstep(L::Q_ARR + ks * 32), kd + dstep(L::K_ARR + L::K_BLK + ks * 32), ID_SH, ks > 0);
 #pragma unroll
                     for (int ks = 0; ks < DT / 32; ++ks)
-                        tc_mma_ss_f8(dt, qd + dstep(KV_BLK + ks * 32), kd + dstep(KV_ARR + ks * 32), ID_SH, 1u);
+                        tc_mma_ss_f8<CG>(dt, qd + dstep(L::Q_ARR + L::Q_BLK + ks * 32), kd + dstep(L::K_ARR + ks * 32), ID_SH, 1u);
                     // + q_h k_h in fp16, the corrections brought back by 2^-12 on the first k-step
 #pragma unroll
                     for (int ks = 0; ks < DT / 16; ++ks) {
-                        const uint32_t bd = kd + dstep((ks >> 2) * KV_BLK + (ks & 3) * 32);
+                        const uint32_t ad = qd + dstep((ks >> 2) * L::Q_BLK + (ks & 3) * 32);
+                        const uint32_t bd = kd + dstep((ks >> 2) * L::K_BLK + (ks & 3) * 32);
                         if (ks == 0)
-                            tc_mma_ts_scaled12(dt, T_Q, bd, ID_SH);
+                            tc_mma_ss_scaled12<CG>(dt, ad, bd, ID_SH);
                         else
-                            tc_mma_ts(dt, T_Q + 8 * ks, bd, ID_SH, 1u);
+                            tc_mma_ss<CG>(dt, ad, bd, ID_SH, 1u);
                     }
                 } else {
-                    // (A, B) pairs: (Q hi, K hi), (Q lo, K hi), (Q hi, K lo); k-steps of 16 over D,
-                    // 16 columns = 32 B inside a 128 B row. The query's high part lives in TMEM
-                    // (16-bit values packed two per column), its low part in shared memory
+                    // (A, B) pairs: (Q hi, K hi), (Q lo, K hi), (Q hi, K lo)
 #pragma unroll
                     for (int prod = 0; prod < (SPLIT ? 3 : 1); ++prod)
 #pragma unroll
-                        for (int ks = 0; ks < DT / 16; ++ks) {
-                            const int koff = (ks >> 2) * KV_BLK + (ks & 3) * 32;
-                            const uint32_t bd = kd + dstep((prod == 2 ? KV_ARR : 0) + koff);
-                            if (prod == 1)
-                                tc_mma_ss(dt, qd + dstep(koff), bd, ID_S, 1u);
-                            else
-                                tc_mma_ts(dt, T_Q + 8 * ks, bd, ID_S, prod > 0 || ks > 0);
-                        }
+                        for (int ks = 0; ks < DT / 16; ++ks)
+                            tc_mma_ss<CG>(dt, qd + dstep((prod == 1 ? L::Q_ARR : 0) + (ks >> 2) * L::Q_BLK + (ks & 3) * 32),
+                                          kd + dstep((prod == 2 ? L::K_ARR : 0) + (ks >> 2) * L::K_BLK + (ks & 3) * 32), ID_S,
+                                          prod > 0 || ks > 0);
                 }
-                tc_commit(sbase + BAR(B_S_FULL + ST));
+                tc_commit<CG>(sbase + BAR(L::B_S_FULL + ST));
             }
             __syncwarp();
         };
-        // value product of a tile of parity ST: P, 128 keys of fp16 values packed two per column,
-        // times V, 64 keys x 128 B rows per block: 16 keys = two 8-row atoms (SBO 1024); the
+        // value product of a tile of ring stage ST: P (in TMEM, the buffer of the tile's parity), 128
+        // keys of fp16 values packed two per column, times V, 64 keys x 128 B rows per block: 16 keys = two 8-row atoms (SBO 1024); the
         // second 64-column block of head dim is LBO = 16 KB away
         auto issue_o = [&](auto st_c, uint32_t acc) {
             constexpr int ST = decltype(st_c)::value;
-            const uint32_t vd = desc_lo(sbase + OFF_V + ST * V_STAGE, KV_BLK);
+            const uint32_t vd = desc_lo(sbase + L::OFF_V + ST * L::V_STAGE, L::V_BLK);
             if (elect_one()) {
 #pragma unroll
                 for (int ks = 0; ks < BN / 16; ++ks)
-                    tc_mma_ts(T_O, T_P + 8 * ks, vd + dstep(ks * 2048), ID_O, ks > 0 ? 1u : acc);
-                tc_commit(sbase + BAR(B_PV_DONE + ST));
+                    tc_mma_ts<CG>(T_O, T_P0 + ST * (BN / 2) + 8 * ks, vd + dstep(ks * 2048), ID_O, ks > 0 ? 1u : acc);
+                tc_commit<CG>(sbase + BAR(L::B_PV_DONE + ST));
             }
             __syncwarp();
         };
@@ -683,39 +793,40 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             return got;
         };
-        // score products of tile j (parity ST) into the buffer that tile j - 2 has been read out of
-        auto next_s = [&](auto st_c, int j) -> bool {
-            constexpr int ST = decltype(st_c)::value;
-            const int par = (j >> 1) & 1;
-            if (!wait_all(B_K_FULL + ST, par)) return false;
-            if (j >= 2 && !wait_all(B_S_READ + ST, par ^ 1)) return false;
-            issue_s(st_c);
-            return true;
+        // the scores of tile j, as soon as those of tile j - 2 have been read out: they are there
+        // when the group of tile j comes for them
+        auto score_step = [&](auto st_c, int j) {
+            if (!ok || j >= n_kt) return;
+            ok = wait_all(L::B_S_GO + decltype(st_c)::value, (j / NSK) & 1);
+            if (ok) issue_s(st_c);
         };
-        // Tile j, parity ST: the scores of tile j + 3 (the other group reads tile j + 1 out while
-        // this one forms P of tile j), so that scores are always there when a group comes for
-        // them; then, with P of tile j written and its values landed (relayed by the loader), its
-        // value product.
-        auto tile_step = [&](auto st_c, auto other_c, int j) {
-            constexpr int ST = decltype(st_c)::value;
-            if (j + 3 < n_kt) ok = next_s(other_c, j + 3);
-            if (!ok) return;
-            ok = wait_all(B_P_FULL + ST, (j >> 1) & 1);
+        auto value_step = [&](auto st_c, int j) {
+            if (!ok || j >= n_kt) return;
+            ok = wait_all(L::B_P_GO + decltype(st_c)::value, (j / NSV) & 1);
             if (ok) issue_o(st_c, j > 0 ? 1u : 0u);
         };
-        constexpr std::integral_constant<int, 0> even{};
-        constexpr std::integral_constant<int, 1> odd{};
-        ok = wait_all(B_Q, 0) && next_s(even, 0);
-        if (ok && n_kt > 1) ok = next_s(odd, 1);
-        if (ok && n_kt > 2) ok = next_s(even, 2);
-        for (int j = 0; j < n_kt && ok; j += 2) {
-            tile_step(even, odd, j);
-            if (ok && j + 1 < n_kt) tile_step(odd, even, j + 1);
+        using I0 = std::integral_constant<int, 0>;
+        using I1 = std::integral_constant<int, 1>;
+        using I2 = std::integral_constant<int, 2>;
+        using I3 = std::integral_constant<int, 3>;
+        if (warp == kScoreWarp) {
+            for (int j = 0; j < n_kt && ok; j += 4) {
+                score_step(I0{}, j);
+                score_step(I1{}, j + 1);
+                score_step(I2{}, j + 2);
+                score_step(I3{}, j + 3);
+            }
+        } else {
+            for (int j = 0; j < n_kt && ok; j += 2) {
+                value_step(I0{}, j);
+                value_step(I1{}, j + 1);
+            }
         }
         // every product issued has to finish before TMEM is released
-        if (elect_one()) tc_commit(sbase + BAR(B_END));
+        const int end = warp == kValueWarp ? L::B_END + 1 : L::B_END;
+        if (elect_one()) tc_commit<CG>(sbase + BAR(end));
         __syncwarp();
-        mbar_wait_own(sbase + BAR(B_END), 0);
+        mbar_wait_own(sbase + BAR(end), 0);
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
@@ -730,38 +841,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
         const float sc = a.scale_log2;
         const float v_absmax = *a.v_absmax;
-        // this thread's half of the query row: the high part into TMEM (OC / 2 packed columns)
-        {
-            const int64_t qrow = ((row_ok ? i : 0) * a.Hq + h) * DT + OC * grp;
-            const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(q_hi) + qrow);
-            uint32_t qw[OC / 2];
-#pragma unroll
-            for (int u = 0; u < OC / 8; ++u) {
-                const uint4 x = row_ok ? src[u] : make_uint4(0u, 0u, 0u, 0u);
-                qw[4 * u] = x.x;
-                qw[4 * u + 1] = x.y;
-                qw[4 * u + 2] = x.z;
-                qw[4 * u + 3] = x.w;
-            }
-            const uint32_t tq = T_Q + lane_off + (OC / 2) * grp;
-#pragma unroll
-            for (int c = 0; c < OC / 2; c += 16) tmem_st16(tq + c, qw + c);
-            if (SPLIT) {
-                // the low part as the K-major A operand in shared memory: 64-column blocks of 128
-                // rows of 128 bytes, 16-byte pieces swizzled by the row
-                src = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(q_lo) + qrow);
-#pragma unroll
-                for (int u = 0; u < OC / 8; ++u) {
-                    const int piece = (OC / 8) * grp + u;
-                    *reinterpret_cast<uint4 *>(smem + OFF_Q + (piece >> 3) * KV_BLK + r * 128 +
-                                               (((piece & 7) ^ (r & 7)) << 4)) =
-                        row_ok ? src[u] : make_uint4(0u, 0u, 0u, 0u);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            }
-            tc_fence_before();
-            mbar_arrive(smem_u32(&bars[B_Q]));
-        }
+        if (lane == 0) arrive_lead(L::B_S_GO + grp);  // the group's score buffer is free for its first tile
         // kept keys of word e of tile j (keys 128 (kt0 + j) + 32 e .. +31): the bitmap's word, or
         // the range suffix_lo .. i (dense: 0 .. i)
         constexpr bool kRange = DENSE || SUFFIX;
@@ -801,9 +881,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t sc2 = f2_pack(sc, sc);
         float l = 0.f, m_own = -INFINITY;  // row sum over this thread's tiles, relative to 2^m_own
         for (int j = grp; j < n_kt; j += 2) {
-            const int par = (j >> 1) & 1;
             if (!kRange) mask_words(j + 4, nnw);
-            if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_S_FULL + grp]), par, wl));
+            if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1, wl));
             tc_fence_after();
             uint32_t su[2][64];
             tmem_issue64(T_S0 + grp * BN + lane_off, su[0]);
@@ -818,7 +897,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             pin64(su[1]);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bars[B_S_READ + grp]));
+            if (lane == 0 && j + 2 < n_kt) arrive_lead(L::B_S_GO + (j + 2) % NSK);
             float sv[BN];
 #pragma unroll
             for (int c = 0; c < BN; ++c) sv[c] = __uint_as_float(su[c >> 6][c & 63]);
@@ -844,9 +923,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             const float mx =
                 fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * sc;
-            // The row's reference maximum moves on from tile to tile, handed to the other group as
-            // soon as it is known. Lazy rescale: it moves, and O is rescaled, only when the row max
-            // grows by more than 2^8. The TMEM loads / stores are warp-collective
+            // The row's reference maximum moves on from tile to tile, handed to the other group. Lazy rescale: it moves, and O is rescaled, only when the row max
+            // grows by more than kLazyLog2. The TMEM loads / stores are warp-collective
             // (.sync.aligned), so the whole warp runs them when any of its rows needs it; the
             // other rows multiply by 1.
             float m_prev = -INFINITY;
@@ -854,34 +932,29 @@ __global__ void __launch_bounds__(kThreads, 1)
                 pair_sync(1 + 2 * wq + (grp ^ 1));
                 m_prev = m_sh[r];
             }
-            const bool upd = mx > m_prev + 8.f;
+            const bool upd = mx > m_prev + kLazyLog2;
             const float m_ref = upd ? mx : m_prev;
-            if (j + 1 < n_kt) {
-                m_sh[r] = m_ref;
-                __threadfence_block();
-                pair_arrive(1 + 2 * wq + grp);
-            }
-            if (!ok) continue;
-            // the value product of tile j - 1 is done: O has settled, and P may be written over
-            auto pv_done = [&]() -> bool {
-                return j == 0 || __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_PV_DONE + (grp ^ 1)]),
-                                                                   ((j - 1) >> 1) & 1, wl));
+            // the value product of tile t is done (t < 0: nothing to wait for)
+            auto pv_done = [&](int t) -> bool {
+                return t < 0 || __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
             };
             const bool scale_o = upd && m_prev != -INFINITY;
-            if (__any_sync(0xFFFFFFFFu, scale_o)) {
-                ok = pv_done();
-                if (!ok) continue;
+            if (ok && __any_sync(0xFFFFFFFFu, scale_o)) {
+                // O has settled once the value product of tile j - 1 is done; that of tile j - 2 first, so
+                // that the barrier is not polled a phase early
+                ok = pv_done(j - 2) && pv_done(j - 1);
                 tc_fence_after();
                 const float al = scale_o ? exp2f(m_prev - m_ref) : 1.f;
 #pragma unroll 1
-                for (int c0 = 0; c0 < DT; c0 += 16) {
-                    float ov[16];
-                    uint32_t ow[16];
-                    tmem_ld16(T_O + lane_off + c0, ov);
+                for (int c0 = 0; c0 < DT && ok; c0 += 32) {
+                    float ov[32];
+                    uint32_t ow[32];
+                    tmem_ld32(T_O + lane_off + c0, ov);
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) ow[c] = __float_as_uint(ov[c] * al);
-                    tmem_st16(T_O + lane_off + c0, ow);
+                    for (int c = 0; c < 32; ++c) ow[c] = __float_as_uint(ov[c] * al);
+                    tmem_st32(T_O + lane_off + c0, ow);
                 }
+                tmem_wait_st();
             }
             if (m_ref != m_own) {
                 l *= m_own == -INFINITY ? 0.f : exp2f(m_own - m_ref);
@@ -894,41 +967,44 @@ __global__ void __launch_bounds__(kThreads, 1)
             // values with slightly perturbed weights).
             uint64_t lsum[2] = {0ull, 0ull};
             const uint64_t nmu2 = f2_pack(-mu, -mu);
+            uint32_t hw[BN / 2];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                uint32_t hw[BN / 4];
-#pragma unroll
-                for (int w = 0; w < BN / 4; ++w) {
-                    const int c = (BN / 2) * half + 2 * w;
-                    float x0, x1;
-                    f2_unpack(f2_fma(f2_pack(sv[c], sv[c + 1]), sc2, nmu2), x0, x1);
-                    const __half2 hp = __floats2half2_rn(ex2(x0), ex2(x1));
-                    const float2 pr = __half22float2(hp);
-                    lsum[w & 1] = f2_add(lsum[w & 1], f2_pack(pr.x, pr.y));
-                    hw[w] = *reinterpret_cast<const uint32_t *>(&hp);
-                }
-                if (half == 0) {
-                    ok = pv_done();
-                    if (!ok) break;
-                    tc_fence_after();
-                }
-                tmem_st32(T_P + lane_off + (BN / 4) * half, hw);
+            for (int w = 0; w < BN / 2; ++w) {
+                float x0, x1;
+                f2_unpack(f2_fma(f2_pack(sv[2 * w], sv[2 * w + 1]), sc2, nmu2), x0, x1);
+                const __half2 hp = __floats2half2_rn(ex2(x0), ex2(x1));
+                const float2 pr = __half22float2(hp);
+                lsum[w & 1] = f2_add(lsum[w & 1], f2_pack(pr.x, pr.y));
+                hw[w] = *reinterpret_cast<const uint32_t *>(&hp);
+            }
+            // Only now on to the other group: its exponentials (the other warp of this scheduler) run
+            // while this warp stores P and takes the next tile's scores and maximum, and not
+            // against this warp's own
+            if (j + 1 < n_kt) {
+                m_sh[r] = m_ref;
+                __threadfence_block();
+                pair_arrive(1 + 2 * wq + grp);
             }
             if (!ok) continue;
+            ok = pv_done(j - 2);  // P's buffer is free
+            if (!ok) continue;
+            tc_fence_after();
+            const uint32_t tp = T_P0 + grp * (BN / 2) + lane_off;
+            tmem_st32(tp, hw);
+            tmem_st32(tp + 32, hw + 32);
             float la, lb;
             f2_unpack(f2_add(lsum[0], lsum[1]), la, lb);
             l += la + lb;
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bars[B_P_FULL + grp]));
+            if (lane == 0) arrive_lead(L::B_P_GO + grp);
         }
         // the row's maximum and sum from both threads
         ml_sh[grp][r] = make_float2(m_own, l);
         ok = !pair_or(9 + wq, !ok);
-        if (ok)
-            ok = __all_sync(0xFFFFFFFFu,
-                            mbar_wait(smem_u32(&bars[B_PV_DONE + ((n_kt - 1) & 1)]), ((n_kt - 1) >> 1) & 1, wl));
+        for (int t = max(0, n_kt - 2); t < n_kt && ok; ++t)  // in order, as above
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
         if (ok) {
             tc_fence_after();
             const float2 ma = ml_sh[0][r], mb = ml_sh[1][r];
@@ -939,19 +1015,34 @@ __global__ void __launch_bounds__(kThreads, 1)
             // fp16 values were scaled by 2^-E for the value product
             const float vs = __uint_as_float((uint32_t)(127 + v_scale_exp(v_absmax)) << 23);
             const float inv = lt > 0.f ? vs / lt : 0.f;
-            TOut *out = SUFFIX ? reinterpret_cast<TOut *>(a.part_o + ((row_ok ? i : 0) * a.Hq + h) * DT + OC * grp)
-                               : reinterpret_cast<TOut *>(a.out) + (((int64_t)s * a.N + (row_ok ? i : 0)) * a.Hq + h) * DT +
-                                     OC * grp;
+            // O, normalised, through shared memory (the ring is free: every load was consumed) so that
+            // neighbouring lanes store neighbouring pieces of a row: stores of 16 bytes per lane and
+            // row took 4,000 cycles of a CTA. A warp's part: its 32 rows x OC columns, 16-byte
+            // pieces swizzled by the row.
+            constexpr int RB = OC * (int)sizeof(TOut), NP = RB / 16;  // bytes and pieces of a row's part
+            unsigned char *stage = smem + warp * (32 * RB);
 #pragma unroll
             for (int c0 = 0; c0 < OC; c0 += 32) {
                 float ov[32];
                 tmem_ld32(T_O + lane_off + OC * grp + c0, ov);
-                if (row_ok) {
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) ov[c] *= inv;
+                for (int c = 0; c < 32; ++c) ov[c] *= inv;
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) store8<TOut>(out + c0 + 8 * e, ov + 8 * e);
+                for (int e = 0; e < 32 * (int)sizeof(TOut) / 16; ++e) {
+                    const int piece = c0 * (int)sizeof(TOut) / 16 + e;
+                    store16<TOut>(stage + lane * RB + ((piece ^ (lane & (NP - 1))) << 4), ov + e * (16 / (int)sizeof(TOut)));
                 }
+            }
+            __syncwarp();
+            const int64_t w0 = q0 + 32 * wq;  // the warp's first row
+            TOut *out = (SUFFIX ? reinterpret_cast<TOut *>(a.part_o) : reinterpret_cast<TOut *>(a.out) + (int64_t)s * a.N * a.Hq * DT) +
+                        (int64_t)h * DT + OC * grp;
+#pragma unroll
+            for (int e = 0; e < NP; ++e) {
+                const int rr = e * (32 / NP) + lane / NP, piece = lane & (NP - 1);
+                const uint4 x = *reinterpret_cast<const uint4 *>(stage + rr * RB + ((piece ^ (rr & (NP - 1))) << 4));
+                if (w0 + rr >= a.row0 && w0 + rr < a.row1)
+                    *reinterpret_cast<uint4 *>(out + (w0 + rr) * a.Hq * DT + piece * (16 / (int)sizeof(TOut))) = x;
             }
             if (SUFFIX) {
                 if (row_ok && grp == 0) a.part_lse[i * a.Hq + h] = m_fin + __log2f(lt);
@@ -962,11 +1053,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 
     if (!ok) atomicOr(&g_ris_tile_error, 2u);
+    __syncwarp();
     tc_fence_before();
+    // CG = 2: neither CTA may leave while the other can still reach its shared memory or TMEM
+    if constexpr (CG == 2) cluster_sync();
     __syncthreads();
     tc_fence_after();
-    if (warp == kMmaWarp)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    if (warp == kScoreWarp) tmem_dealloc<CG>(tmem);
 }
 
 // ---------------------------------------------------------------- host side
@@ -1001,7 +1094,7 @@ bool make_map3(CUtensorMap *m, const void *base, int64_t N, int H, int rows, int
 }
 
 template <int DT, bool SPLIT, bool DENSE, typename TOut, bool SUFFIX = false>
-cudaError_t launch_t(const AttnArgs &a, const TileMaps &maps, const void *q_hi, const void *q_lo, cudaStream_t s)
+cudaError_t launch_t(const AttnArgs &a, const TileMaps &maps, cudaStream_t s)
 {
     auto kern = k_attn_tile<DT, SPLIT, DENSE, SUFFIX, TOut>;
     static bool attr = false;
@@ -1015,9 +1108,23 @@ cudaError_t launch_t(const AttnArgs &a, const TileMaps &maps, const void *q_hi, 
         if (fa.numRegs < kRegs) return cudaErrorInvalidConfiguration;
         attr = true;
     }
+    constexpr int CG = Lay<DT>::CG;
     const int64_t n_qt = (a.row1 + BM - 1) / BM - a.row0 / BM;  // tiles covering rows row0 .. row1-1
-    const unsigned grid = (unsigned)(n_qt * a.Hq * a.n_sets);
-    kern<<<grid, kThreads, SMEM_BYTES, s>>>(a, maps, q_hi, q_lo);
+    const bool tile_pair = CG == 2 && (a.G & 1) != 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((tile_pair ? (n_qt + 1) / 2 * 2 : n_qt) * a.Hq * a.n_sets));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CG;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, maps);
+    if (e != cudaSuccess) return e;
     note_launch();
     return cudaGetLastError();
 }
@@ -1036,31 +1143,37 @@ cudaError_t read_tile_error(unsigned int *out)
     return cudaMemcpyToSymbol(g_ris_tile_error, &zero, sizeof(unsigned int));
 }
 
-// K / V tensor maps of a call (the key low part only with split queries and keys; the values
-// as fp16).
-bool make_maps(TileMaps &maps, const AttnArgs &a, bool split, int D)
+// Q / K / V tensor maps of a call (the low parts only with split queries and keys; the values
+// as fp16). q_hi, q_lo: moved back by a.q_first rows, as the kernels' other row pointers.
+bool make_maps(TileMaps &maps, const AttnArgs &a, const void *q_hi, const void *q_lo, int D)
 {
+    const bool split = q_lo != nullptr;
     if (a.v16 == nullptr || a.v_absmax == nullptr) return false;
-    if (!make_map3(&maps.kh, a.k, a.N, a.Hkv, BN, D) || !make_map3(&maps.v, a.v16, a.N, a.Hkv, BN, D, true)) return false;
-    if (split) return make_map3(&maps.kl, a.k_lo, a.N, a.Hkv, BN, D);
+    const int krows = D == 128 ? Lay<128>::KROWS : Lay<64>::KROWS;  // keys of a box
+    if (!make_map3(&maps.kh, a.k, a.N, a.Hkv, krows, D) || !make_map3(&maps.v, a.v16, a.N, a.Hkv, BN, D, true)) return false;
+    const size_t back = (size_t)a.q_first * a.Hq * D * 2;
+    auto q_map = [&](CUtensorMap *m, const void *q) {
+        return make_map3(m, static_cast<const char *>(q) + back, a.q_rows, a.Hq, BM, D);
+    };
+    if (!q_map(&maps.qh, q_hi)) return false;
+    if (split) return q_map(&maps.ql, q_lo) && make_map3(&maps.kl, a.k_lo, a.N, a.Hkv, krows, D);
     maps.kl = maps.kh;
+    maps.ql = maps.qh;
     return true;
 }
 
 template <int DT>
-cudaError_t launch_tile_d(const AttnArgs &a, const TileMaps &maps, const void *q_hi, const void *q_lo, int out_dtype,
-                          bool dense, cudaStream_t s)
+cudaError_t launch_tile_d(const AttnArgs &a, const TileMaps &maps, bool split, int out_dtype, bool dense, cudaStream_t s)
 {
-    const bool split = q_lo != nullptr;
     if (out_dtype == RIS_F32) {
-        if (split) return dense ? launch_t<DT, true, true, float>(a, maps, q_hi, q_lo, s) : launch_t<DT, true, false, float>(a, maps, q_hi, q_lo, s);
-        return dense ? launch_t<DT, false, true, float>(a, maps, q_hi, q_lo, s) : launch_t<DT, false, false, float>(a, maps, q_hi, q_lo, s);
+        if (split) return dense ? launch_t<DT, true, true, float>(a, maps, s) : launch_t<DT, true, false, float>(a, maps, s);
+        return dense ? launch_t<DT, false, true, float>(a, maps, s) : launch_t<DT, false, false, float>(a, maps, s);
     }
     if (split)
-        return dense ? launch_t<DT, true, true, __nv_bfloat16>(a, maps, q_hi, q_lo, s)
-                     : launch_t<DT, true, false, __nv_bfloat16>(a, maps, q_hi, q_lo, s);
-    return dense ? launch_t<DT, false, true, __nv_bfloat16>(a, maps, q_hi, q_lo, s)
-                 : launch_t<DT, false, false, __nv_bfloat16>(a, maps, q_hi, q_lo, s);
+        return dense ? launch_t<DT, true, true, __nv_bfloat16>(a, maps, s)
+                     : launch_t<DT, true, false, __nv_bfloat16>(a, maps, s);
+    return dense ? launch_t<DT, false, true, __nv_bfloat16>(a, maps, s)
+                 : launch_t<DT, false, false, __nv_bfloat16>(a, maps, s);
 }
 
 // q_hi / q_lo: queries as a bf16 pair [N][Hq][D] (q_lo null: exact bf16 queries and keys,
@@ -1072,9 +1185,9 @@ cudaError_t launch_attention_tile(const AttnArgs &a, int D, const void *q_hi, co
     std::lock_guard<std::mutex> lk(mu);
     if (D != 128 && D != 64) return cudaErrorInvalidValue;
     alignas(64) TileMaps maps;
-    if (!make_maps(maps, a, q_lo != nullptr, D)) return cudaErrorInvalidValue;
-    return D == 128 ? launch_tile_d<128>(a, maps, q_hi, q_lo, out_dtype, dense, s)
-                    : launch_tile_d<64>(a, maps, q_hi, q_lo, out_dtype, dense, s);
+    if (!make_maps(maps, a, q_hi, q_lo, D)) return cudaErrorInvalidValue;
+    return D == 128 ? launch_tile_d<128>(a, maps, q_lo != nullptr, out_dtype, dense, s)
+                    : launch_tile_d<64>(a, maps, q_lo != nullptr, out_dtype, dense, s);
 }
 
 cudaError_t launch_attention_tile_suffix(const AttnArgs &a, int D, const void *q_hi, const void *q_lo, cudaStream_t s)
@@ -1085,12 +1198,12 @@ cudaError_t launch_attention_tile_suffix(const AttnArgs &a, int D, const void *q
         return cudaErrorInvalidValue;
     const bool split = q_lo != nullptr;
     alignas(64) TileMaps maps;
-    if (!make_maps(maps, a, split, D)) return cudaErrorInvalidValue;
+    if (!make_maps(maps, a, q_hi, q_lo, D)) return cudaErrorInvalidValue;
     if (D == 128)
-        return split ? launch_t<128, true, false, float, true>(a, maps, q_hi, q_lo, s)
-                     : launch_t<128, false, false, float, true>(a, maps, q_hi, q_lo, s);
-    return split ? launch_t<64, true, false, float, true>(a, maps, q_hi, q_lo, s)
-                 : launch_t<64, false, false, float, true>(a, maps, q_hi, q_lo, s);
+        return split ? launch_t<128, true, false, float, true>(a, maps, s)
+                     : launch_t<128, false, false, float, true>(a, maps, s);
+    return split ? launch_t<64, true, false, float, true>(a, maps, s)
+                 : launch_t<64, false, false, float, true>(a, maps, s);
 }
 
 }  // namespace ris

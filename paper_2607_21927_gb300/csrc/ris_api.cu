@@ -752,6 +752,8 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
     a.debug_no_loads = g_tile_no_loads.load(std::memory_order_relaxed);
     a.row0 = row0;
     a.row1 = row1;
+    a.q_first = q_first;
+    a.q_rows = q_rows;
     a.n_tasks = (int64_t)a.n_sets * (row1 - row0) * kv_heads;
     a.qk_bound = tile8 ? (const float *)bound.p : nullptr;
     if (tile || suffix || tile8) {

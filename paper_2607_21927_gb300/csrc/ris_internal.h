@@ -89,6 +89,8 @@ struct AttnArgs {
     int32_t n_sets;        // output sets: n_seeds for per-seed masks, else 1
     int64_t row0;          // query rows row0 .. row1-1 are computed (0 and N for a whole layer)
     int64_t row1;
+    int64_t q_first;       // first row that q (before it was moved back by these rows) holds, and how
+    int64_t q_rows;        // many: 0 and N, or the row range of a call on local rows
     // Dense-suffix split (part_o set): every key in [lo(i), i] of row i is kept, lo(i) being
     // the start of the row's Structural block of clique_B tokens (0: no blocks) and / or of its
     // forced local window of `window` keys, whichever reaches further back. The tile kernel's
