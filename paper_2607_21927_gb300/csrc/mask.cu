@@ -5,9 +5,10 @@
 // causal bitmap row with all seeds OR-merged in registers (the paper's streaming merge,
 // without ever holding a seed's mask), then compacted into ascending per-row key lists.
 //
-//   k_mask_bits : per (mask, row) CTA, per 32-key word: Philox4x32-10 draws of every seed
-//                 (8 calls = 32 keys per seed), OR, forced window/anchors, Structural
-//                 block clique, causal cut; writes the word and the row's key count.
+//   k_mask_bits : per (mask, row) CTA, per group of 4 keys: one Philox4x32-10 call per seed, the
+//                 smallest word over the seeds against the threshold, then per 32-key word the
+//                 forced window/anchors, Structural block clique and causal cut; writes the
+//                 word and the row's key count.
 //   k_mask_draws: index-draw sampler only: per (mask, row) CTA, the row's index draws of
 //                 every seed (one Philox call = 4 draws), j = floor(u N / 2^32), kept when
 //                 j < i by an atomic OR into the zeroed bitmap row; k_mask_bits then ORs the
@@ -41,18 +42,9 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
     return c;
 }
 
-__device__ __forceinline__ uint32_t bits_below(int64_t n)  // bits [0, n) set, n in [0, 32]
-{
-    return n >= 32 ? 0xFFFFFFFFu : (n <= 0 ? 0u : ((1u << n) - 1u));
-}
-
-// Set bits for keys [lo, hi] (inclusive) inside the word holding keys [j0, j0 + 32).
-__device__ __forceinline__ uint32_t range_bits(int64_t j0, int64_t lo, int64_t hi)
-{
-    if (hi < lo) return 0u;
-    const int64_t a = lo - j0, b = hi - j0 + 1;  // [a, b) relative to j0
-    return bits_below(b) & ~bits_below(a);
-}
+// bits of a word at and above / at and below bit x (any x)
+__device__ __forceinline__ uint32_t bits_from(int x) { return x <= 0 ? 0xFFFFFFFFu : x > 31 ? 0u : 0xFFFFFFFFu << x; }
+__device__ __forceinline__ uint32_t bits_to(int x) { return x >= 31 ? 0xFFFFFFFFu : x < 0 ? 0u : 0xFFFFFFFFu >> (31 - x); }
 
 __device__ __forceinline__ int64_t row_word_offset(int64_t i)
 {
@@ -62,63 +54,132 @@ __device__ __forceinline__ int64_t row_word_offset(int64_t i)
 
 constexpr int kBitsThreads = 128;
 
-__global__ void __launch_bounds__(kBitsThreads) k_mask_bits(const MaskBitsArgs a)
-{
-    // rows are visited from the last (longest) to the first
-    const int64_t r = (int64_t)blockIdx.x;
-    const int32_t m = (int32_t)(r % a.n_masks);
-    const bool one = a.single_row >= 0;
-    const int64_t i = one ? a.single_row : a.N - 1 - r / a.n_masks;
-    const uint32_t head_key = (a.heads_keyed > 1) ? (uint32_t)(m % a.heads_keyed) : 0u;
-    const int32_t s0 = a.per_seed ? m / a.heads_keyed : 0;
-    const int32_t s1 = a.per_seed ? s0 + 1 : a.n_seeds;
-    const int64_t nw = (i >> 5) + 1;
-    uint32_t *row = a.bitmap + (int64_t)m * a.words_per_mask + (one ? 0 : row_word_offset(i));
-    const int64_t blk0 = (a.mode == RIS_MODE_STRUCTURAL) ? (i / a.B) * a.B : i + 1;
+// What the draws of one (mask, row) share: the row's counter words and the head key's schedule.
+struct RowDraws {
+    uint32_t i, layer, k1;  // counter word 1, counter word 3, key word 1
+    uint32_t s_hi, s_lo;    // the product of round 1 on counter word 2 (the stream)
+};
 
-    int64_t count = 0;
-    for (int64_t w = threadIdx.x; w < nw; w += kBitsThreads) {
-        const int64_t j0 = w << 5;
-        // forced keys: local window (i-W, i], anchors [0, A), Structural clique [blk0, i]
-        uint32_t bits = a.or_existing ? row[w] : 0u;
-        bits |= range_bits(j0, i - a.W + 1, i);
-        bits |= range_bits(j0, 0, (int64_t)a.A - 1);
-        bits |= range_bits(j0, blk0, i);
-        const uint32_t causal = range_bits(j0, 0, i - 1);  // drawn pairs are j < i
-        if (a.thr > 0) {
-            // u < thr for thr in [1, 2^32] is u <= thr - 1 in 32 bits
-            const uint32_t tm1 = a.thr > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)(a.thr - 1);
-#pragma unroll 1
-            for (int32_t s = s0; s < s1; ++s) {
-                const uint32_t seed = a.seeds.v[s];
+// Smallest word over the seeds s0 .. s1-1 of each of the 4 keys of the groups g .. g + U - 1 (keys
+// 4 g .. 4 g + 4 U - 1): a key is kept by some seed iff this minimum is below the threshold.
+//
+// Philox4x32-10 as in philox4x32_10 above, with what the 10 rounds of a row's calls have in common
+// taken out of the loop over seeds. Round 1 multiplies the group (word 0) and the stream (word 2),
+// neither of which depends on the seed; its results z, w depend on the group only (key word 1 is
+// the head key) and x, y on the row and seed only. So the second product of round 2 depends on the
+// group only and the first on the seed only: per call 8 rounds of two products remain, 16 of 20.
+template <int U, int SEEDS>
+__device__ __forceinline__ void min_words(const MaskBitsArgs &a, const RowDraws &d, uint32_t g, int s0, int s1,
+                                          uint32_t (&best)[U][4])
+{
+    uint32_t hx[U], y2[U], wz[U];  // x2 but for key word 0, y2, z2 but for the seed's product
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint32_t need = (causal >> (4 * c)) & ~(bits >> (4 * c)) & 0xFu;
-                    if (need == 0) continue;
-                    const uint4 u = philox4x32_10(
-                        make_uint4((uint32_t)((j0 >> 2) + c), (uint32_t)i, a.stream, a.layer_key),
-                        seed, head_key);
-                    uint32_t keep = 0;
-                    keep |= (u.x <= tm1) ? 1u : 0u;
-                    keep |= (u.y <= tm1) ? 2u : 0u;
-                    keep |= (u.z <= tm1) ? 4u : 0u;
-                    keep |= (u.w <= tm1) ? 8u : 0u;
-                    bits |= (keep & need) << (4 * c);
-                }
+    for (int u = 0; u < U; ++u) {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * (g + u);
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * ((uint32_t)(p0 >> 32) ^ d.layer ^ d.k1);
+        hx[u] = (uint32_t)(p1 >> 32) ^ d.s_lo;
+        y2[u] = (uint32_t)p1;
+        wz[u] = (uint32_t)p0 ^ (d.k1 + 0xBB67AE85u);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) best[u][e] = 0xFFFFFFFFu;
+    }
+#pragma unroll SEEDS
+    for (int s = s0; s < s1; ++s) {
+        uint32_t k0 = a.seeds.v[s], k1 = d.k1 + 0xBB67AE85u;
+        const uint64_t ps = (uint64_t)0xD2511F53u * (d.s_hi ^ d.i ^ k0);
+        k0 += 0x9E3779B9u;
+        uint4 c[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            c[u] = make_uint4(hx[u] ^ k0, y2[u], (uint32_t)(ps >> 32) ^ wz[u], (uint32_t)ps);
+#pragma unroll
+        for (int r = 2; r < 10; ++r) {
+            k0 += 0x9E3779B9u;
+            k1 += 0xBB67AE85u;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint64_t p0 = (uint64_t)0xD2511F53u * c[u].x;
+                const uint64_t p1 = (uint64_t)0xCD9E8D57u * c[u].z;
+                c[u] = make_uint4((uint32_t)(p1 >> 32) ^ c[u].y ^ k0, (uint32_t)p1,
+                                  (uint32_t)(p0 >> 32) ^ c[u].w ^ k1, (uint32_t)p0);
             }
         }
-        bits &= range_bits(j0, 0, one ? i - 1 : i);  // a single row keeps keys j < i only
-        row[w] = bits;
-        count += __popc(bits);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            best[u][0] = min(best[u][0], c[u].x);
+            best[u][1] = min(best[u][1], c[u].y);
+            best[u][2] = min(best[u][2], c[u].z);
+            best[u][3] = min(best[u][3], c[u].w);
+        }
+    }
+}
+
+// One CTA per (mask, row), one warp per 16 words (512 keys) at a time: lane l takes the 16 keys of
+// half a word, groups 4 l .. 4 l + 3 of the step's 128, and its neighbour the other half.
+//
+// Bound by the 32 x 32 -> 64-bit products (32 lanes per clock and SM, a quarter of the fp32 rate)
+// and, nearly as much, by the ALU pipe (an exclusive or per product, the minima, the key schedule).
+// MANY: two seeds per loop pass and as many registers as the compiler wants (the key schedules stay in
+// registers); else eight CTAs per SM, for masks of one or two seeds, where a row's other work
+// counts. Measured at N = 16384 of 1% (few / many): 1 seed 138 / 144 us, 2 217 / 217, 3 297 / 283, 8 693 /
+// 641, 20 1644 / 1487. 70 seeds at N = 32768: 29.0 ms with every round in the loop over seeds and one
+// thread per word, 21.1 with rounds 1 and 2 taken out, 19.6 now (1.5 calls per clock and SM).
+constexpr int kManySeeds = 3;
+template <bool MANY>
+__global__ void __launch_bounds__(kBitsThreads, MANY ? 1 : 8) k_mask_bits(const MaskBitsArgs a)
+{
+    // rows are visited from the last (longest) to the first
+    const uint32_t m = blockIdx.x % (uint32_t)a.n_masks;
+    const bool one = a.single_row >= 0;
+    const int i = (int)(one ? a.single_row : a.N - 1 - blockIdx.x / (uint32_t)a.n_masks);  // below 2^31
+    const int32_t s0 = a.per_seed ? (int)m / a.heads_keyed : 0;
+    const int32_t s1 = a.per_seed ? s0 + 1 : a.n_seeds;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *row = a.bitmap + (int64_t)m * a.words_per_mask + (one ? 0 : row_word_offset(i));
+    // forced keys: local window (i-W, i], anchors [0, A), Structural clique [block start, i]; the draws
+    // matter for j < i before the first and the last
+    int tail0 = i - a.W + 1;
+    if (a.mode == RIS_MODE_STRUCTURAL) tail0 = min(tail0, (int)((uint32_t)i / (uint32_t)a.B * (uint32_t)a.B));
+    const int last = one ? i - 1 : i;  // a single row keeps keys j < i only
+    const int nw = (i >> 5) + 1;
+    const int ng = a.thr > 0 ? (max(0, min(i, tail0)) + 3) >> 2 : 0;
+    // u < thr for thr in [1, 2^32] is u <= thr - 1 in 32 bits
+    const uint32_t tm1 = a.thr > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)(a.thr - 1);
+    RowDraws d;
+    d.i = (uint32_t)i;
+    d.layer = a.layer_key;
+    d.k1 = (a.heads_keyed > 1) ? m % (uint32_t)a.heads_keyed : 0u;
+    const uint64_t ps = (uint64_t)0xCD9E8D57u * a.stream;
+    d.s_hi = (uint32_t)(ps >> 32);
+    d.s_lo = (uint32_t)ps;
+
+    int count = 0;
+    for (int w0 = 16 * warp; w0 < nw; w0 += 16 * (kBitsThreads / 32)) {
+        uint32_t word = 0u;
+        if (8 * w0 < ng) {
+            uint32_t best[4][4];
+            min_words<4, MANY ? 2 : 1>(a, d, (uint32_t)(8 * w0 + 4 * lane), s0, s1, best);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) word |= best[e >> 2][e & 3] <= tm1 ? 1u << e : 0u;
+        }
+        word |= __shfl_down_sync(0xFFFFFFFFu, word, 1) << 16;
+        const int w = w0 + (lane >> 1);
+        if ((lane & 1) == 0 && w < nw) {
+            const int j0 = w << 5;
+            uint32_t bits = word & bits_to(i - 1 - j0);  // drawn pairs are j < i
+            if (a.or_existing) bits |= row[w];
+            bits = (bits | bits_from(tail0 - j0) | bits_to(a.A - 1 - j0)) & bits_to(last - j0);
+            row[w] = bits;
+            count += __popc(bits);
+        }
     }
     // block reduction of the row count
-    __shared__ int64_t red[kBitsThreads / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xFFFFFFFFu, count, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = count;
+    __shared__ int red[kBitsThreads / 32];
+    count = __reduce_add_sync(0xFFFFFFFFu, count);
+    if (lane == 0) red[warp] = count;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int64_t t = 0;
+        int t = 0;  // a row holds at most 2^31 - 1 keys
 #pragma unroll
         for (int k = 0; k < kBitsThreads / 32; ++k) t += red[k];
         a.counts[one ? (int64_t)m : (int64_t)m * a.N + i] = t;
@@ -287,7 +348,10 @@ __global__ void __launch_bounds__(kFillThreads) k_mask_fill(const MaskFillArgs a
 cudaError_t launch_mask_bits(const MaskBitsArgs &a, cudaStream_t s)
 {
     const int64_t blocks = (int64_t)a.n_masks * (a.single_row >= 0 ? 1 : a.N);
-    k_mask_bits<<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
+    if ((a.per_seed ? 1 : a.n_seeds) >= kManySeeds)
+        k_mask_bits<true><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
+    else
+        k_mask_bits<false><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
     note_launch();
     return cudaGetLastError();
 }

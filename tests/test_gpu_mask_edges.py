@@ -1,0 +1,24 @@
+"""Mask sampler at the edges of its steps: rows around one word and around a warp's 512 keys, odd and
+even seed counts on both sides of the few / many line, windows and anchors at their extremes."""
+import numpy as np
+import pytest
+
+from paper_2607_21927_gb300 import ris
+from test_gpu_mask import check_rows, gpu_mask, oracle_spec
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N", [2, 31, 64, 511, 514, 2050])
+@pytest.mark.parametrize("S", [1, 2, 3, 5])
+@pytest.mark.parametrize("mode,W,A,head_keyed,sampler", [
+    (0, 1, 0, False, 0), (1, 1, 5, True, 0), (0, 2**31 - 1, 0, False, 0), (0, 1, 2**31 - 1, False, 0),
+    (1, 700, 33, False, ris.SAMPLER_DRAWS)])
+def test_mask_steps(N, S, mode, W, A, head_keyed, sampler):
+    seeds = [11 + 7 * s for s in range(S)]
+    m = gpu_mask(N, mode, 0.07, seeds, kv_heads=2, W=W, A=A, per_head=head_keyed, layer_key=3, sampler=sampler)
+    heads = range(2) if head_keyed else [0]
+    specs = [oracle_spec(N, mode, 0.07, seeds, W=min(W, N), A=min(A, N), head_key=h, layer_key=3, sampler=sampler)
+             for h in heads]
+    rows = np.unique(np.clip([0, 1, 30, 31, 32, 510, 511, 512, 513, 2047, 2048, 2049, N - 2, N - 1], 0, N - 1))
+    check_rows(m, specs, rows)
