@@ -702,7 +702,8 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
             pa.Hq = heads;
             pa.Hkv = kv_heads;
             pa.D = head_dim;
-            std::memcpy(pa.f, ra.f, sizeof(pa.f));
+            for (int c = 0; c < head_dim / 2; ++c)  // f <= 1: below a sixth of a turn per position
+                pa.turn[c] = (uint64_t)(ra.f[c] * (18446744073709551616.0 / 6.283185307179586476925286766559));
             pa.mscale = ra.mscale;
             RIS_CUDA(launch_fp8_prep(pa, s));
         } else {

@@ -177,7 +177,7 @@ unsigned int read_decode_error();
 cudaError_t launch_rope(const RopeArgs &a, int dtype_in, int dtype_out, cudaStream_t s);
 
 // The pre-passes of a layer call whose scores take the fp8-correction operands (see
-// fp8_score_scales in attn_common.cuh), bf16 inputs, head dim a multiple of 16, every pointer
+// fp8_score_scales in attn_common.cuh), bf16 inputs, head dim 128, every pointer
 // 16-byte aligned. Two launches: bounds of |q~|, |k~| (and max |v| when v16 is set) into
 // bounds[0..2] (zeroed by this call), then RoPE of q (positions q_first .. q_first + q_rows - 1)
 // and k (positions 0 .. N-1) into q_hi / q_lo and k_hi / k_lo: fp16 hi parts, and per (token,
@@ -191,7 +191,7 @@ struct Fp8PrepArgs {
     float *bounds;          // [3]
     int64_t N, q_rows, q_first;
     int32_t Hq, Hkv, D;
-    double f[kMaxHeadDimHalf];  // rotation frequencies (fp64)
+    uint64_t turn[kMaxHeadDimHalf];  // rotation frequencies as fractions of a turn, in 2^-64
     float mscale;
 };
 cudaError_t launch_fp8_prep(const Fp8PrepArgs &a, cudaStream_t s);

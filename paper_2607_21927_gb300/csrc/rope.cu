@@ -13,6 +13,7 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "attn_common.cuh"
@@ -37,6 +38,7 @@ __device__ __forceinline__ void st_f<__nv_bfloat16>(__nv_bfloat16 *p, float x) {
 
 constexpr int kRopeTokens = 4;   // tokens per CTA (blockDim.y) of k_rope
 constexpr int kPrepTokens = 32;  // tokens per CTA (blockDim.y) of k_fp8_rotate
+constexpr int kPrepDim = 128;    // head dim of the fp8 operands
 
 template <typename TIn, typename TOut, bool LO>
 __global__ void k_rope(const RopeArgs a)
@@ -70,11 +72,11 @@ __global__ void k_rope(const RopeArgs a)
     }
 }
 
-// largest squared pair norm over the 8 pairs (c + e, c + e + D/2), e < 8, of a bf16 row
-__device__ __forceinline__ float pair_norm2_max8(const __nv_bfloat16 *row, int c, int half)
+// largest squared pair norm over the 8 pairs (e, e + D/2), e < 8, from x on
+__device__ __forceinline__ float pair_norm2_max8(const __nv_bfloat16 *x)
 {
-    const uint4 a = *reinterpret_cast<const uint4 *>(row + c);
-    const uint4 b = *reinterpret_cast<const uint4 *>(row + c + half);
+    const uint4 a = *reinterpret_cast<const uint4 *>(x);
+    const uint4 b = *reinterpret_cast<const uint4 *>(x + kPrepDim / 2);
     const uint32_t wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
     float m = 0.f;
 #pragma unroll
@@ -89,41 +91,48 @@ __device__ __forceinline__ float pair_norm2_max8(const __nv_bfloat16 *row, int c
 // Pass 1 of the fp8-operand pre-passes: bounds[0] / bounds[1] = mscale times the largest pair
 // norm of q / k, with a margin of 2^-20 for the rotation's fp32 rounding (a rotation keeps
 // every pair's norm, so these bound every rotated value), bounds[2] = max |v| (when v16 is
-// set). One grid-stride pass over the three tensors in 16-byte pieces (8 pairs of a row, or 8
-// values), one atomic per warp and bound; the bounds are >= 0, so the order of their bit
-// patterns is the order of the values.
-__global__ void k_fp8_bounds(const Fp8PrepArgs a)
+// set). Grid-stride passes over the three tensors in 16-byte pieces (8 pairs of a row, or 8
+// values), one atomic per CTA and bound: one per warp, 29,000 to the same three words, took longer
+// than the reads of a short sequence (23 us at N = 3001). The bounds are >= 0, so the order of their
+// bit patterns is the order of the values.
+constexpr int kBoundThreads = 256, kBoundBlocks = 152 * 8;
+__global__ void __launch_bounds__(kBoundThreads) k_fp8_bounds(const Fp8PrepArgs a)
 {
-    const int half = a.D >> 1, per_row = half / 8;
-    const int64_t nq = a.q_rows * a.Hq * per_row, nk = a.N * a.Hkv * per_row;
-    const int64_t nv = a.v16 != nullptr ? a.N * a.Hkv * (a.D / 8) : 0;
-    const __nv_bfloat16 *q = reinterpret_cast<const __nv_bfloat16 *>(a.q);
-    const __nv_bfloat16 *k = reinterpret_cast<const __nv_bfloat16 *>(a.k);
-    float mq = 0.f, mk = 0.f, mv = 0.f;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nq + nk + nv;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        if (t < nq) {
-            const int64_t r = t / per_row;
-            mq = fmaxf(mq, pair_norm2_max8(q + r * a.D, 8 * (int)(t - r * per_row), half));
-        } else if (t < nq + nk) {
-            const int64_t u = t - nq, r = u / per_row;
-            mk = fmaxf(mk, pair_norm2_max8(k + r * a.D, 8 * (int)(u - r * per_row), half));
-        } else {
-            const uint4 x = reinterpret_cast<const uint4 *>(a.v)[t - nq - nk];
+    constexpr int P = kPrepDim / 16;  // pieces of a q / k row
+    const int64_t t0 = (int64_t)blockIdx.x * kBoundThreads + threadIdx.x, step = (int64_t)gridDim.x * kBoundThreads;
+    float m[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int which = 0; which < 2; ++which) {
+        const __nv_bfloat16 *x = reinterpret_cast<const __nv_bfloat16 *>(which == 0 ? a.q : a.k);
+        const int64_t n = (which == 0 ? a.q_rows * a.Hq : a.N * a.Hkv) * P;
+#pragma unroll 2
+        for (int64_t t = t0; t < n; t += step) m[which] = fmaxf(m[which], pair_norm2_max8(x + (t / P) * kPrepDim + 8 * (t % P)));
+    }
+    if (a.v16 != nullptr) {
+        const int64_t n = a.N * a.Hkv * (kPrepDim / 8);
+#pragma unroll 2
+        for (int64_t t = t0; t < n; t += step) {
+            const uint4 x = reinterpret_cast<const uint4 *>(a.v)[t];
             const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                mv = fmaxf(mv, fmaxf(fabsf(__uint_as_float(w[e] << 16)), fabsf(__uint_as_float(w[e] & 0xFFFF0000u))));
+                m[2] = fmaxf(m[2], fmaxf(fabsf(__uint_as_float(w[e] << 16)), fabsf(__uint_as_float(w[e] & 0xFFFF0000u))));
         }
     }
-    mq = sqrtf(warp_max(mq)) * a.mscale * (1.f + 0x1p-20f);
-    mk = sqrtf(warp_max(mk)) * a.mscale * (1.f + 0x1p-20f);
-    mv = warp_max(mv);
-    if ((threadIdx.x & 31) == 0) {
-        unsigned int *b = reinterpret_cast<unsigned int *>(a.bounds);
-        atomicMax(b, __float_as_uint(mq));
-        atomicMax(b + 1, __float_as_uint(mk));
-        if (a.v16 != nullptr) atomicMax(b + 2, __float_as_uint(mv));
+    __shared__ float red[3][kBoundThreads / 32];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        m[k] = warp_max(m[k]);
+        if ((threadIdx.x & 31) == 0) red[k][threadIdx.x >> 5] = m[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int k = threadIdx.x;
+        float x = red[k][0];
+#pragma unroll
+        for (int w = 1; w < kBoundThreads / 32; ++w) x = fmaxf(x, red[k][w]);
+        if (k < 2) x = sqrtf(x) * a.mscale * (1.f + 0x1p-20f);
+        if (k < 2 || a.v16 != nullptr) atomicMax(reinterpret_cast<unsigned int *>(a.bounds) + k, __float_as_uint(x));
     }
 }
 
@@ -140,16 +149,17 @@ __device__ __forceinline__ uint2 to_e4m3x8(const float *x)
     return make_uint2(w[0], w[1]);
 }
 
-// Rotate the 8 pairs (c + e, c + e + D/2), e < 8, of each of H heads of one token (bf16 in) and
+// Rotate the 8 pairs (c + e, c + e + D/2), e < 8, of heads h0 .. h1 - 1 of one token (bf16 in) and
 // write them in the tile kernel's form: fp16 hi parts to hi and, in the 2D-byte record of
 // each (token, head) in lo, e4m3(hi s_hi) at bytes [0, D) and e4m3((y - hi) s_lo) at [D, 2D);
 // or (f8 false) the bf16 hi / lo pair.
-__device__ __forceinline__ void rotate_heads8(const __nv_bfloat16 *x, void *hi, void *lo, int H, int D, int c,
+__device__ __forceinline__ void rotate_heads8(const __nv_bfloat16 *x, void *hi, void *lo, int h0, int h1, int c,
                                               const float *cs, const float *sn, float mscale, bool f8, float s_hi,
                                               float s_lo)
 {
-    const int half = D >> 1;
-    for (int h = 0; h < H; ++h) {
+    constexpr int D = kPrepDim, half = D / 2;
+#pragma unroll 2
+    for (int h = h0; h < h1; ++h) {
         const uint4 a = *reinterpret_cast<const uint4 *>(x + (int64_t)h * D + c);
         const uint4 b = *reinterpret_cast<const uint4 *>(x + (int64_t)h * D + c + half);
         const uint32_t wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
@@ -197,41 +207,55 @@ __device__ __forceinline__ void rotate_heads8(const __nv_bfloat16 *x, void *hi, 
     }
 }
 
-// Pass 2: one thread per (token p, frequencies 8j .. 8j+7): the eight rotation angles (fp64,
-// reduced as in k_rope), then the keys of the token, its query row if it has one (rows q_first
-// .. q_first + q_rows - 1), and, when v16 is set, elements 16j .. 16j+15 of each of its value
-// heads as fp16 scaled by 2^-E (E = v_scale_exp(max |v|)). Queries: hi parts scaled by 2^-ea, lo
-// parts by 2^(12+eb); keys: 2^-eb and 2^(12+ea) (fp8_score_scales).
-__global__ void k_fp8_rotate(const Fp8PrepArgs a)
+// sin and cos of position p times a frequency given as a fraction of a turn in 2^-64 (a.turn): the
+// low 64 bits of the product are the fraction of the turn, signed, exact but for the frequency's own
+// rounding (p 2^-65 of a turn, below the fp64 product's); then 2 pi in fp32 with the
+// fraction's top 24 bits exact and the rest as a correction, one rounding of the angle in
+// effect. The fp64 product and reduction of k_rope run at two operations per clock and SM.
+__device__ __forceinline__ void sincos_turns(uint32_t p, uint64_t turn, float *sn, float *cs)
 {
+    const int64_t frac = (int64_t)(turn * p);
+    const float top = (float)(int32_t)(frac >> 40), rest = (float)(uint32_t)(frac >> 8);
+    constexpr float A = 0x1.921fb6p-22f, A_LO = -0x1.777a5cp-47f, B = 0x1.921fb6p-54f;  // 2 pi 2^-24 (hi, lo), 2 pi 2^-56
+    sincosf(fmaf(top, A, fmaf(top, A_LO, rest * B)), sn, cs);
+}
+
+// Pass 2: one thread per (token p, frequencies 8j .. 8j+7, slice of the heads): the eight rotation
+// angles, then its slice of the Hkv key heads (with elements 16j .. 16j+15 of their value heads as
+// fp16 scaled by 2^-E, E = v_scale_exp(max |v|), when v16 is set) and Hq query heads (of rows
+// q_first .. q_first + q_rows - 1). Queries: hi parts scaled by 2^-ea, lo parts by 2^(12+eb); keys:
+// 2^-eb and 2^(12+ea) (fp8_score_scales). The heads are sliced (gridDim.y) where the tokens alone
+// leave SMs without a CTA.
+__global__ void __launch_bounds__(kPrepDim / 16 * kPrepTokens) k_fp8_rotate(const Fp8PrepArgs a)
+{
+    constexpr int D = kPrepDim;
     const int j = threadIdx.x, c = 8 * j;  // blockDim.x == D / 16
     const int64_t p = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     if (p >= a.N) return;
+    const int heads = a.Hkv + a.Hq, slices = gridDim.y, z = blockIdx.y;
+    const int lo_h = (int)((int64_t)heads * z / slices), hi_h = (int)((int64_t)heads * (z + 1) / slices);
+    const int k0 = min(lo_h, a.Hkv), k1 = min(hi_h, a.Hkv), q0 = max(lo_h - a.Hkv, 0), q1 = max(hi_h - a.Hkv, 0);
+    const bool q_row = p >= a.q_first && p < a.q_first + a.q_rows;
+    if (k0 == k1 && !(q_row && q0 < q1)) return;
     int ea = 0, eb = 0;
     const bool f8 = fp8_score_scales(a.bounds[0], a.bounds[1], ea, eb);
     float cs[8], sn[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        const double ang = (double)p * a.f[c + e];
-        const double n = rint(ang * 0.15915494309189533577);
-        double red = fma(-n, 6.28318530717958623200, ang);
-        red = fma(-n, 2.4492935982947064e-16, red);
-        sincosf((float)red, &sn[e], &cs[e]);
-    }
-    const int64_t hk = p * (int64_t)a.Hkv * a.D;
+    for (int e = 0; e < 8; ++e) sincos_turns((uint32_t)p, a.turn[c + e], &sn[e], &cs[e]);
+    const int64_t hk = p * (int64_t)a.Hkv * D;
     rotate_heads8(reinterpret_cast<const __nv_bfloat16 *>(a.k) + hk, reinterpret_cast<__half *>(a.k_hi) + hk,
-                  reinterpret_cast<unsigned char *>(a.k_lo) + 2 * hk, a.Hkv, a.D, c, cs, sn, a.mscale, f8,
+                  reinterpret_cast<unsigned char *>(a.k_lo) + 2 * hk, k0, k1, c, cs, sn, a.mscale, f8,
                   f8 ? pow2i(-eb) : 1.f, f8 ? pow2i(12 + ea) : 1.f);
-    if (p >= a.q_first && p < a.q_first + a.q_rows) {
-        const int64_t hq = (p - a.q_first) * (int64_t)a.Hq * a.D;
+    if (q_row) {
+        const int64_t hq = (p - a.q_first) * (int64_t)a.Hq * D;
         rotate_heads8(reinterpret_cast<const __nv_bfloat16 *>(a.q) + hq, reinterpret_cast<__half *>(a.q_hi) + hq,
-                      reinterpret_cast<unsigned char *>(a.q_lo) + 2 * hq, a.Hq, a.D, c, cs, sn, a.mscale, f8,
+                      reinterpret_cast<unsigned char *>(a.q_lo) + 2 * hq, q0, q1, c, cs, sn, a.mscale, f8,
                       f8 ? pow2i(-ea) : 1.f, f8 ? pow2i(12 + eb) : 1.f);
     }
     if (a.v16 != nullptr) {
         const float scale = pow2i(-v_scale_exp(a.bounds[2]));
-        for (int h = 0; h < a.Hkv; ++h) {
-            const int64_t e0 = hk + (int64_t)h * a.D + 16 * j;
+        for (int h = k0; h < k1; ++h) {
+            const int64_t e0 = hk + (int64_t)h * D + 16 * j;
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const uint4 x = *reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(a.v) + e0 + 8 * u);
@@ -249,9 +273,9 @@ __global__ void k_fp8_rotate(const Fp8PrepArgs a)
     }
 }
 
-// max |v| over 8 bf16 values per thread and step (grid-stride), one atomic per warp; |v| >= 0,
+// max |v| over 8 bf16 values per thread and step (grid-stride), one atomic per CTA; |v| >= 0,
 // so the order of the float bit patterns is the order of the values
-__global__ void k_absmax_bf16(const uint4 *v, int64_t n8, unsigned int *vmax)
+__global__ void __launch_bounds__(kBoundThreads) k_absmax_bf16(const uint4 *v, int64_t n8, unsigned int *vmax)
 {
     float m = 0.f;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n8; t += (int64_t)gridDim.x * blockDim.x) {
@@ -263,8 +287,15 @@ __global__ void k_absmax_bf16(const uint4 *v, int64_t n8, unsigned int *vmax)
             m = fmaxf(m, fabsf(__uint_as_float(w[k] & 0xFFFF0000u)));
         }
     }
+    __shared__ float red[kBoundThreads / 32];
     m = warp_max(m);
-    if ((threadIdx.x & 31) == 0) atomicMax(vmax, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < kBoundThreads / 32; ++w) m = fmaxf(m, red[w]);
+        atomicMax(vmax, __float_as_uint(m));
+    }
 }
 
 __global__ void k_values_f16(const uint4 *v, int64_t n8, const float *vmax, uint4 *v16)
@@ -288,16 +319,16 @@ __global__ void k_values_f16(const uint4 *v, int64_t n8, const float *vmax, uint
 
 cudaError_t launch_fp8_prep(const Fp8PrepArgs &a, cudaStream_t s)
 {
-    if ((a.D % 16) != 0 || a.D / 2 > kMaxHeadDimHalf || a.D / 16 * kPrepTokens > 1024) return cudaErrorInvalidValue;
+    if (a.D != kPrepDim) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(a.bounds, 0, 3 * sizeof(float), s);
     if (e != cudaSuccess) return e;
-    const int64_t pieces = (a.q_rows * a.Hq + a.N * a.Hkv) * (a.D / 16) + (a.v16 != nullptr ? a.N * a.Hkv * (a.D / 8) : 0);
-    const int threads = 256;
-    const int64_t need = (pieces + threads - 1) / threads;
-    const unsigned grid = (unsigned)(need < 152 * 8 ? (need > 0 ? need : 1) : 152 * 8);
-    k_fp8_bounds<<<grid, threads, 0, s>>>(a);
-    const dim3 block(a.D / 16, kPrepTokens);
-    k_fp8_rotate<<<(unsigned)((a.N + kPrepTokens - 1) / kPrepTokens), block, 0, s>>>(a);
+    const int64_t pieces = a.q_rows * a.Hq * (a.D / 16);  // of the largest tensor
+    const int64_t need = (pieces + kBoundThreads - 1) / kBoundThreads;
+    k_fp8_bounds<<<(unsigned)std::min<int64_t>(std::max<int64_t>(need, 1), kBoundBlocks), kBoundThreads, 0, s>>>(a);
+    // at least six CTAs per SM, as far as there are heads to slice
+    const int64_t blocks = (a.N + kPrepTokens - 1) / kPrepTokens;
+    const int64_t slices = std::min<int64_t>(a.Hq + a.Hkv, std::max<int64_t>(1, (6 * 152 + blocks - 1) / blocks));
+    k_fp8_rotate<<<dim3((unsigned)blocks, (unsigned)slices), dim3(a.D / 16, kPrepTokens), 0, s>>>(a);
     note_launch(2);
     return cudaGetLastError();
 }
@@ -308,7 +339,7 @@ cudaError_t launch_values_f16(const void *v, int64_t n, void *v16, float *vmax, 
     const int64_t n8 = n / 8;
     cudaError_t e = cudaMemsetAsync(vmax, 0, sizeof(float), s);
     if (e != cudaSuccess) return e;
-    const int threads = 256;
+    const int threads = kBoundThreads;
     const int64_t need = (n8 + threads - 1) / threads;
     const unsigned grid = (unsigned)(need < 152 * 8 ? (need > 0 ? need : 1) : 152 * 8);
     k_absmax_bf16<<<grid, threads, 0, s>>>(reinterpret_cast<const uint4 *>(v), n8, reinterpret_cast<unsigned int *>(vmax));
