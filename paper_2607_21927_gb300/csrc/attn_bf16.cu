@@ -255,11 +255,7 @@ __device__ __forceinline__ int velem(int j, int p)
     return (WIDE && D == 128) ? 16 * p + 2 * j : 64 * (j >> 2) + 8 * p + 2 * (j & 3);
 }
 
-constexpr float kLazyLog2 = 8.f;  // rescale O only when the row maximum grows by more than 2^8
-
-#ifndef RIS_ATTN_MIN_BLOCKS
-#define RIS_ATTN_MIN_BLOCKS 1
-#endif
+constexpr float kLazyLog2 = 14.f;  // rescale O only when the row maximum grows by more than 2^14 (P in fp16's range)
 
 // D: head dim (64 or 128). QSPLIT: q is fp32 (split hi + lo); else q is bf16.
 // KSPLIT: keys come as a bf16 hi (a.k) + lo (a.k_lo) pair. WIDE: 32-byte loads (K, K lo and
@@ -591,17 +587,18 @@ __device__ __forceinline__ void gather_task(const AttnArgs &a, int eb, uint32_t 
         // ---- online softmax; lane holds keys p, p+8 x heads 2q, 2q+1
         float s0 = val0 ? s[0] * sc : -INFINITY, s1 = val0 ? s[1] * sc : -INFINITY;
         float s2 = val1 ? s[2] * sc : -INFINITY, s3 = val1 ? s[3] * sc : -INFINITY;
-        float mx0 = fmaxf(s0, s2), mx1 = fmaxf(s1, s3);
-#pragma unroll
-        for (int off = 4; off < 32; off <<= 1) {
-            mx0 = fmaxf(mx0, __shfl_xor_sync(0xFFFFFFFFu, mx0, off));
-            mx1 = fmaxf(mx1, __shfl_xor_sync(0xFFFFFFFFu, mx1, off));
-        }
         // Lazy rescaling: the reference maximum only moves when a score exceeds it by more
         // than 2^kLazyLog2 (probabilities then stay below 2^kLazyLog2 and the fp32 sums stay
-        // exact enough), so most groups skip the rescale of O; the branch is warp-uniform.
-        const bool need0 = mx0 > m0 + kLazyLog2, need1 = mx1 > m1 + kLazyLog2;
-        if (__any_sync(0xFFFFFFFFu, need0 || need1)) {
+        // exact enough), so most groups skip the rescale of O, and the row maximum over the lanes with
+        // it: a vote on the lanes' own scores tells. The branch is warp-uniform.
+        float mx0 = fmaxf(s0, s2), mx1 = fmaxf(s1, s3);
+        if (__any_sync(0xFFFFFFFFu, mx0 > m0 + kLazyLog2 || mx1 > m1 + kLazyLog2)) {
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) {
+                mx0 = fmaxf(mx0, __shfl_xor_sync(0xFFFFFFFFu, mx0, off));
+                mx1 = fmaxf(mx1, __shfl_xor_sync(0xFFFFFFFFu, mx1, off));
+            }
+            const bool need0 = mx0 > m0 + kLazyLog2, need1 = mx1 > m1 + kLazyLog2;
             const float mn0 = need0 ? mx0 : m0, mn1 = need1 ? mx1 : m1;
             const float al0 = need0 ? exp2f(m0 - mn0) : 1.f, al1 = need1 ? exp2f(m1 - mn1) : 1.f;
             m0 = mn0;
@@ -728,12 +725,14 @@ __device__ __forceinline__ void gather_task(const AttnArgs &a, int eb, uint32_t 
 
 // F8: the queries and keys came from launch_fp8_prep; which of its two schemes it wrote
 // follows from the bounds at a.qk_bound, read here on the device as it did.
+// Head dim 64 with bf16 key pairs: four CTAs per SM instead of three, at 36 bytes of spills (32 / 4
+// heads, N = 16384, 5.8% of the pairs: layer call 1,135 -> 1,066 us; five, at 308 bytes, 1,549).
 // F8: the query fragments and output accumulators live in tensor memory
 // (each thread's own TMEM lane, 128 columns per CTA), which leaves room for three CTAs of four
 // warps per SM instead of two, and so more gathered rows in flight.
 constexpr int kGatherTmemCols = 128;
 template <int D, bool QSPLIT, bool KSPLIT, bool WIDE, typename TIdx, bool DENSE, typename TOut, bool SEEDS, bool F8>
-__global__ void __launch_bounds__(kAttnWarps * 32, F8 ? 3 : RIS_ATTN_MIN_BLOCKS) k_attn_bf16(const AttnArgs a)
+__global__ void __launch_bounds__(kAttnWarps * 32, F8 ? 3 : D == 64 && QSPLIT ? (SEEDS ? 3 : 4) : 1) k_attn_bf16(const AttnArgs a)
 {
     if constexpr (F8) {
         __shared__ uint32_t tbase_sh;

@@ -192,16 +192,20 @@ const char *forced_design()
 }
 
 
-// Union density at and above which masked dense tiles beat gathering pair by pair (bf16,
-// head dim 128): a tile costs the dense causal products (an fp16 score product, two e4m3 score
-// corrections and one value product) whatever the mask, a gathered pair 1.25 KB of K/V rows.
-// Measured crossover on Qwen2-shaped layers (head dim 128): 6.8% of the causal pairs at
-// N = 65536 and N = 32768 (tiles 13.25 / 3.34 ms per launch; the gather on the fp8 operands
-// 11.38 / 2.89 ms at 5.85%, 13.15 / 3.33 ms at 6.8%); on TinyLlama-shaped layers (head dim 64, 32 query and 4 KV
-// heads, N = 16384, three bf16 score products) 11.1% (tiles 1.94 ms, the gather 1.69 / 1.99 ms
-// at 9.6% / 11.4%), where the tiles are half the products but the same softmax work.
-constexpr double kTileDensity = 0.068;
-constexpr double kTileDensity64 = 0.111;
+// Union density at and above which masked dense tiles beat gathering pair by pair (bf16): a tile
+// costs the dense causal products whatever the mask, a gathered pair 1.25 KB of K/V rows (head dim 128
+// with the fp8 operands). Measured kernel times per launch, gather / tiles, where they cross:
+//   head dim 128, 12 / 2 heads  N = 4096 60 / 64 us at 4.9%, 66 / 64 at 5.9%; 8192 180 / 198, 207 / 198;
+//                               16384 619 / 671, 723 / 671; 32768 2.31 / 2.70 ms, 2.73 / 2.69;
+//                               65536 9.06 / 10.46 ms at 4.9%, 10.7 / 11.0 at 5.9%, 12.4 / 11.0 at 6.8%
+//   head dim 64, 32 / 4 heads   N = 8192 373 / 421 us at 7.7%, 451 / 420 at 9.6%; 16384 1.38 / 1.53 ms, 1.68 / 1.55;
+//                               32768 5.32 / 6.02 ms, 6.55 / 5.95
+// Below 3072 tokens the tiles' clusters no longer fill the SMs evenly (N = 2048: 31 / 33 us at 7.8%, 33 / 32 at
+// 9.6%; N = 1024: 16 / 18 us at 11.5%; head dim 64, N = 2048: 45 / 52 us at 11.4%), and the line rises as the
+// sequence shortens, to 13% (20% at head dim 64) below 1365 tokens.
+constexpr double kTileDensity = 0.058;
+constexpr double kTileDensity64 = 0.088;
+double tile_line_factor(int64_t N) { return std::min(2.25, std::max(1.0, 3072.0 / (double)N)); }
 
 // Shortest dense span (Structural block or local window) for which the split pays: two
 // 128-key tiles.
@@ -258,7 +262,8 @@ int design_of(const ris_mask_s *m, int32_t dtype, int32_t head_dim, int32_t grou
     if (tiles) {
         const double causal = (double)m->n_masks * ((double)m->N * (double)(m->N + 1) / 2.0);
         const double gathered = (double)m->n_pairs - (split ? (double)m->n_masks * (double)m->suffix_pairs : 0.0);
-        if (gathered >= (head_dim == 64 ? kTileDensity64 : kTileDensity) * causal) return 2;
+        const double line = (head_dim == 64 ? kTileDensity64 : kTileDensity) * tile_line_factor(m->N);
+        if (gathered >= line * causal) return 2;
     }
     return split ? 4 : 0;
 }
