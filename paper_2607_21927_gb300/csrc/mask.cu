@@ -14,7 +14,7 @@
 //                 j < i by an atomic OR into the zeroed bitmap row; k_mask_bits then ORs the
 //                 forced and clique keys into those words and counts the row.
 //   k_scan_*    : exclusive scan of the counts into row_ptr (int64).
-//   k_mask_fill : per (mask, row) CTA, expands the bitmap row into ascending key indices.
+//   k_mask_fill : per (mask, row) warp, expands the bitmap row into ascending key indices.
 //
 // Integer-only; every decision is an exact comparison of a 32-bit word with a host-resolved
 // 64-bit threshold, so the result is bit-exact across devices and hosts.
@@ -247,6 +247,37 @@ __device__ __forceinline__ int64_t block_inclusive(int64_t v, int64_t *smem)
     return v;
 }
 
+// In-place inclusive scan of x[0, n) by one CTA, tile after tile: one launch where the three below
+// would have a tile or two (n = 3001: 4.8 us instead of 10; four tiles, 14.8 us, are as slow).
+constexpr int64_t kScanOneTiles = 2;
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(int64_t *x, int64_t n)
+{
+    __shared__ int64_t smem[32];
+    __shared__ int64_t total;
+    int64_t carry = 0;
+    for (int64_t t0 = 0; t0 < n; t0 += kScanTile) {
+        const int64_t base = t0 + (int64_t)threadIdx.x * kScanPer;
+        int64_t vals[kScanPer];
+        int64_t sum = 0;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            vals[e] = (base + e < n) ? x[base + e] : 0;
+            sum += vals[e];
+        }
+        const int64_t incl = block_inclusive(sum, smem);
+        int64_t run = carry + incl - sum;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            run += vals[e];
+            if (base + e < n) x[base + e] = run;
+        }
+        if (threadIdx.x == kScanThreads - 1) total = incl;
+        __syncthreads();
+        carry += total;
+        __syncthreads();
+    }
+}
+
 // In-place inclusive scan of each tile of x[0, n); tile totals to partials[tile].
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(int64_t *x, int64_t n, int64_t *partials)
 {
@@ -299,22 +330,25 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_add(int64_t *x, int64_t n
 // ---------------------------------------------------------------- CSR fill
 constexpr int kFillThreads = 128;
 
+// One warp per (mask, row), a word per lane and step, the next step's words in flight meanwhile. (A CTA
+// per row, with two barriers per 128 words, took 79 us for ten one-seed masks of N = 8192.)
 template <typename TIdx>
-__global__ void __launch_bounds__(kFillThreads) k_mask_fill(const MaskFillArgs a)
+__global__ void __launch_bounds__(kFillThreads) k_mask_fill(const MaskFillArgs a, int64_t n_tasks)
 {
-    __shared__ int64_t warp_tot[kFillThreads / 32];
-    const int64_t r = (int64_t)blockIdx.x;
-    const int32_t m = (int32_t)(r % a.n_masks);
+    const int64_t r = (int64_t)blockIdx.x * (kFillThreads / 32) + (threadIdx.x >> 5);
+    if (r >= n_tasks) return;
+    const uint32_t m = (uint32_t)r % (uint32_t)a.n_masks;  // below 2^31
     const bool one = a.single_row >= 0;
-    const int64_t i = one ? a.single_row : a.N - 1 - r / a.n_masks;
-    const int64_t nw = (i >> 5) + 1;
+    const int64_t i = one ? a.single_row : a.N - 1 - (uint32_t)r / (uint32_t)a.n_masks;
+    const int nw = (int)(i >> 5) + 1;
     const uint32_t *row = a.bitmap + (int64_t)m * a.words_per_mask + (one ? 0 : row_word_offset(i));
     TIdx *col = reinterpret_cast<TIdx *>(a.col) + a.row_ptr[one ? (int64_t)m : (int64_t)m * a.N + i];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int64_t carry = 0;
-    for (int64_t w0 = 0; w0 < nw; w0 += kFillThreads) {
-        const int64_t w = w0 + threadIdx.x;
-        uint32_t bits = w < nw ? row[w] : 0u;
+    const int lane = threadIdx.x & 31;
+    uint32_t next = lane < nw ? row[lane] : 0u;
+    for (int w0 = 0; w0 < nw; w0 += 32) {
+        const int w = w0 + lane;
+        uint32_t bits = next;
+        next = w + 32 < nw ? row[w + 32] : 0u;
         const int c = __popc(bits);
         int incl = c;
 #pragma unroll
@@ -322,24 +356,12 @@ __global__ void __launch_bounds__(kFillThreads) k_mask_fill(const MaskFillArgs a
             const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
             if (lane >= o) incl += t;
         }
-        if (lane == 31) warp_tot[warp] = incl;
-        __syncthreads();
-        int64_t before = carry;
-        int64_t chunk = 0;
-#pragma unroll
-        for (int k = 0; k < kFillThreads / 32; ++k) {
-            if (k < warp) before += warp_tot[k];
-            chunk += warp_tot[k];
-        }
-        int64_t pos = before + incl - c;
-        const int64_t j0 = w << 5;
+        TIdx *dst = col + (incl - c);
         while (bits) {
-            const int b = __ffs(bits) - 1;
-            col[pos++] = (TIdx)(j0 + b);
+            *dst++ = (TIdx)((w << 5) + __ffs(bits) - 1);
             bits &= bits - 1;
         }
-        carry += chunk;
-        __syncthreads();
+        col += __shfl_sync(0xFFFFFFFFu, incl, 31);
     }
 }
 
@@ -369,6 +391,11 @@ int64_t scan_partials_count(int64_t n) { return (n + kScanTile - 1) / kScanTile;
 cudaError_t launch_scan_inplace(int64_t *x, int64_t n, int64_t *partials, cudaStream_t s)
 {
     const int64_t tiles = scan_partials_count(n);
+    if (tiles <= kScanOneTiles) {
+        k_scan_one<<<1, kScanThreads, 0, s>>>(x, n);
+        note_launch();
+        return cudaGetLastError();
+    }
     k_scan_tiles<<<(unsigned)tiles, kScanThreads, 0, s>>>(x, n, partials);
     k_scan_partials<<<1, kScanThreads, 0, s>>>(partials, tiles);
     k_scan_add<<<(unsigned)tiles, kScanThreads, 0, s>>>(x, n, partials);
@@ -378,11 +405,12 @@ cudaError_t launch_scan_inplace(int64_t *x, int64_t n, int64_t *partials, cudaSt
 
 cudaError_t launch_mask_fill(const MaskFillArgs &a, cudaStream_t s)
 {
-    const int64_t blocks = (int64_t)a.n_masks * (a.single_row >= 0 ? 1 : a.N);
+    const int64_t tasks = (int64_t)a.n_masks * (a.single_row >= 0 ? 1 : a.N);
+    const unsigned blocks = (unsigned)((tasks + kFillThreads / 32 - 1) / (kFillThreads / 32));
     if (a.col_bytes == 2)
-        k_mask_fill<uint16_t><<<(unsigned)blocks, kFillThreads, 0, s>>>(a);
+        k_mask_fill<uint16_t><<<blocks, kFillThreads, 0, s>>>(a, tasks);
     else
-        k_mask_fill<uint32_t><<<(unsigned)blocks, kFillThreads, 0, s>>>(a);
+        k_mask_fill<uint32_t><<<blocks, kFillThreads, 0, s>>>(a, tasks);
     note_launch();
     return cudaGetLastError();
 }
