@@ -669,12 +669,11 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
     const void *qu = q, *ku = k, *kl = nullptr, *q_lo = nullptr;
     bool q_split = false;
     if (rotated) {
-        RopeArgs ra{};
-        double ms = 1.0;
-        RIS_TRY(ris_rope_freqs(rope, N, head_dim, ra.f, &ms));
-        ra.N = N;
-        ra.D = head_dim;
-        ra.mscale = (float)ms;
+        double f[kMaxHeadDimHalf], ms = 1.0;
+        uint64_t turn[kMaxHeadDimHalf] = {};
+        RIS_TRY(ris_rope_freqs(rope, N, head_dim, f, &ms));
+        for (int c = 0; c < head_dim / 2; ++c)  // f <= 1: below a sixth of a turn per position
+            turn[c] = (uint64_t)(f[c] * (18446744073709551616.0 / 6.283185307179586476925286766559));
         const size_t nq = (size_t)q_rows * heads * head_dim, nk = (size_t)N * kv_heads * head_dim;
         // rotated queries: fp32 (split into bf16 hi + lo by the gather kernels) or a 16-bit pair
         // (the fp8 scheme's operands, or a bf16 hi + lo pair); rotated keys in fp32, or for bf16
@@ -707,25 +706,26 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
             pa.Hq = heads;
             pa.Hkv = kv_heads;
             pa.D = head_dim;
-            for (int c = 0; c < head_dim / 2; ++c)  // f <= 1: below a sixth of a turn per position
-                pa.turn[c] = (uint64_t)(ra.f[c] * (18446744073709551616.0 / 6.283185307179586476925286766559));
-            pa.mscale = ra.mscale;
+            std::memcpy(pa.turn, turn, sizeof(turn));
+            pa.mscale = (float)ms;
             RIS_CUDA(launch_fp8_prep(pa, s));
         } else {
-            ra.x_in = q;
-            ra.x_out = qt.p;
-            ra.x_out_lo = q_pair ? qtl.p : nullptr;
-            ra.H = heads;
-            ra.N = q_rows;
-            ra.pos0 = q_first;
-            RIS_CUDA(launch_rope(ra, dtype, q_pair ? RIS_BF16 : RIS_F32, s));
+            RopeQkArgs ra{};
+            ra.q = q;
+            ra.k = k;
+            ra.q_out = qt.p;
+            ra.q_lo = qtl.p;
+            ra.k_out = kt.p;
+            ra.k_lo = ktl.p;
             ra.N = N;
-            ra.pos0 = 0;
-            ra.x_in = k;
-            ra.x_out = kt.p;
-            ra.x_out_lo = ktl.p;
-            ra.H = kv_heads;
-            RIS_CUDA(launch_rope(ra, dtype, dtype, s));
+            ra.q_rows = q_rows;
+            ra.q_first = q_first;
+            ra.Hq = heads;
+            ra.Hkv = kv_heads;
+            ra.D = head_dim;
+            std::memcpy(ra.turn, turn, sizeof(turn));
+            ra.mscale = (float)ms;
+            RIS_CUDA(launch_rope_qk(ra, dtype, s));
         }
         qu = back(qt.p, (size_t)heads * head_dim * (q_pair ? 2 : 4));
         q_lo = back(qtl.p, (size_t)heads * head_dim * 2);

@@ -176,6 +176,19 @@ unsigned int read_decode_error();
 // dtype_in / dtype_out are ris_dtype values.
 cudaError_t launch_rope(const RopeArgs &a, int dtype_in, int dtype_out, cudaStream_t s);
 
+// RoPE of q (rows at positions q_first .. q_first + q_rows - 1) and k (positions 0 .. N-1) of a layer
+// call in one launch, every pointer 16-byte aligned, D a multiple of 16. fp32 inputs: q_out and k_out
+// fp32. bf16 inputs: k_out / k_lo a bf16 hi / lo pair, q_out / q_lo likewise, or q_out fp32 with q_lo null.
+struct RopeQkArgs {
+    const void *q, *k;
+    void *q_out, *q_lo, *k_out, *k_lo;
+    int64_t N, q_rows, q_first;
+    int32_t Hq, Hkv, D;
+    uint64_t turn[kMaxHeadDimHalf];  // rotation frequencies as fractions of a turn, in 2^-64
+    float mscale;
+};
+cudaError_t launch_rope_qk(const RopeQkArgs &a, int dtype, cudaStream_t s);
+
 // The pre-passes of a layer call whose scores take the fp8-correction operands (see
 // fp8_score_scales in attn_common.cuh), bf16 inputs, head dim 128, every pointer
 // 16-byte aligned. Two launches: bounds of |q~|, |k~| (and max |v| when v16 is set) into

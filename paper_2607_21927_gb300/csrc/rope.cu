@@ -273,6 +273,92 @@ __global__ void __launch_bounds__(kPrepDim / 16 * kPrepTokens) k_fp8_rotate(cons
     }
 }
 
+// Eight bf16 or four fp32 values of a 16-byte piece as fp32.
+__device__ __forceinline__ void unpack16(const uint4 &x, float (&o)[8], const __nv_bfloat16 *)
+{
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        o[2 * e] = __uint_as_float(w[e] << 16);
+        o[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u);
+    }
+}
+__device__ __forceinline__ void unpack16(const uint4 &x, float (&o)[4], const float *)
+{
+    o[0] = __uint_as_float(x.x);
+    o[1] = __uint_as_float(x.y);
+    o[2] = __uint_as_float(x.z);
+    o[3] = __uint_as_float(x.w);
+}
+
+// V rotated values to fp32, or (PAIR) to a bf16 hi part and the residual of its rounding.
+template <bool PAIR, int V>
+__device__ __forceinline__ void store_rotated(void *hi, void *lo, int64_t at, const float (&y)[V])
+{
+    if constexpr (PAIR) {
+        uint32_t wh[V / 2], wl[V / 2];
+#pragma unroll
+        for (int e = 0; e < V; e += 2) {
+            const __nv_bfloat162 hb = __floats2bfloat162_rn(y[e], y[e + 1]);
+            const float2 hv = __bfloat1622float2(hb);
+            const __nv_bfloat162 lb = __floats2bfloat162_rn(y[e] - hv.x, y[e + 1] - hv.y);
+            wh[e / 2] = *reinterpret_cast<const uint32_t *>(&hb);
+            wl[e / 2] = *reinterpret_cast<const uint32_t *>(&lb);
+        }
+        static_assert(V == 8, "16-byte stores of a pair");
+        *reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(hi) + at) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
+        *reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(lo) + at) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < V; e += 4)
+            *reinterpret_cast<float4 *>(static_cast<float *>(hi) + at + e) = make_float4(y[e], y[e + 1], y[e + 2], y[e + 3]);
+    }
+}
+
+// RoPE of a layer call's q and k in one launch: one thread per (token, V frequencies of a 16-byte
+// piece, slice of the heads), sliced as k_fp8_rotate's. fp32 inputs come out in fp32, bf16 keys as a
+// bf16 hi / lo pair, bf16 queries as a pair (QPAIR) or in fp32. Two launches of k_rope, with one element
+// per thread and load, took 20 + 10 us for 12 / 2 fp32 heads of 128 at N = 6007 and 50 + 13 us for 32 / 4
+// bf16 heads of 64 at N = 16384.
+template <typename T, bool QPAIR>
+__global__ void __launch_bounds__(256) k_rope_qk(const RopeQkArgs a)
+{
+    constexpr int V = 16 / (int)sizeof(T);
+    constexpr bool KPAIR = sizeof(T) == 2;
+    const int half = a.D >> 1, c = V * threadIdx.x;  // blockDim.x == half / V
+    const int64_t p = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+    if (p >= a.N) return;
+    const int heads = a.Hkv + a.Hq, slices = gridDim.y, z = blockIdx.y;
+    const int lo_h = (int)((int64_t)heads * z / slices), hi_h = (int)((int64_t)heads * (z + 1) / slices);
+    const bool q_row = p >= a.q_first && p < a.q_first + a.q_rows;
+    if (lo_h >= a.Hkv && !q_row) return;
+    float cs[V], sn[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) sincos_turns((uint32_t)p, a.turn[c + e], &sn[e], &cs[e]);
+#pragma unroll 2
+    for (int hh = lo_h; hh < hi_h; ++hh) {
+        const bool key = hh < a.Hkv;
+        if (!key && !q_row) break;
+        const int64_t at = key ? (p * a.Hkv + hh) * a.D + c : ((p - a.q_first) * a.Hq + (hh - a.Hkv)) * a.D + c;
+        const T *x = static_cast<const T *>(key ? a.k : a.q) + at;
+        float x0[V], x1[V], y0[V], y1[V];
+        unpack16(*reinterpret_cast<const uint4 *>(x), x0, (const T *)nullptr);
+        unpack16(*reinterpret_cast<const uint4 *>(x + half), x1, (const T *)nullptr);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            y0[e] = fmaf(x0[e], cs[e], -x1[e] * sn[e]) * a.mscale;
+            y1[e] = fmaf(x1[e], cs[e], x0[e] * sn[e]) * a.mscale;
+        }
+        if (key) {
+            store_rotated<KPAIR, V>(a.k_out, a.k_lo, at, y0);
+            store_rotated<KPAIR, V>(a.k_out, a.k_lo, at + half, y1);
+        } else {
+            store_rotated<QPAIR, V>(a.q_out, a.q_lo, at, y0);
+            store_rotated<QPAIR, V>(a.q_out, a.q_lo, at + half, y1);
+        }
+    }
+}
+
 // max |v| over 8 bf16 values per thread and step (grid-stride), one atomic per CTA; |v| >= 0,
 // so the order of the float bit patterns is the order of the values
 __global__ void __launch_bounds__(kBoundThreads) k_absmax_bf16(const uint4 *v, int64_t n8, unsigned int *vmax)
@@ -330,6 +416,24 @@ cudaError_t launch_fp8_prep(const Fp8PrepArgs &a, cudaStream_t s)
     const int64_t slices = std::min<int64_t>(a.Hq + a.Hkv, std::max<int64_t>(1, (6 * 152 + blocks - 1) / blocks));
     k_fp8_rotate<<<dim3((unsigned)blocks, (unsigned)slices), dim3(a.D / 16, kPrepTokens), 0, s>>>(a);
     note_launch(2);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rope_qk(const RopeQkArgs &a, int dtype, cudaStream_t s)
+{
+    const int V = dtype == RIS_BF16 ? 8 : 4, x = a.D / 2 / V;
+    if (a.D % (2 * V) != 0 || x > 256 || (dtype == RIS_F32 && a.q_lo != nullptr)) return cudaErrorInvalidValue;
+    const dim3 block((unsigned)x, (unsigned)(256 / x));
+    const int64_t blocks = (a.N + block.y - 1) / block.y;
+    const int64_t slices = std::min<int64_t>(a.Hq + a.Hkv, std::max<int64_t>(1, (6 * 152 + blocks - 1) / blocks));
+    const dim3 grid((unsigned)blocks, (unsigned)slices);
+    if (dtype == RIS_F32)
+        k_rope_qk<float, false><<<grid, block, 0, s>>>(a);
+    else if (a.q_lo != nullptr)
+        k_rope_qk<__nv_bfloat16, true><<<grid, block, 0, s>>>(a);
+    else
+        k_rope_qk<__nv_bfloat16, false><<<grid, block, 0, s>>>(a);
+    note_launch();
     return cudaGetLastError();
 }
 
