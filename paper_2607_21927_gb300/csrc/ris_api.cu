@@ -462,9 +462,34 @@ ris_status ris_rope_freqs(const ris_rope_cfg *rope, int64_t N, int32_t head_dim,
     return RIS_OK;
 }
 
-ris_status ris_mask_generate(int64_t N, int32_t kv_heads, int32_t mode, double density, const uint32_t *seeds,
+}  // extern "C"
+
+namespace {
+
+// Expected pairs of all masks of a call: the forced keys, and the others with the probability that one
+// of a mask's seeds draws them.
+double expected_pairs(const ris_mask_s *m, const ris_mask_opts &o)
+{
+    const double n = (double)m->N, causal = n * (n + 1.0) / 2.0;
+    const ris_params &p = m->params;
+    const double hit = o.sampler == 1 ? 1.0 - std::pow(1.0 - 1.0 / n, (double)p.draws) : (double)p.thr / 4294967296.0;
+    const int64_t block = m->mode == RIS_MODE_STRUCTURAL ? p.block : 0;
+    const double anchors = std::min((double)o.n_anchor, n);
+    const double forced = std::min(causal, (double)suffix_pairs_of(m->N, block, o.local_window) +
+                                               anchors * std::max(0.0, n - std::max<double>(o.local_window, (double)block)));
+    return m->n_masks * (forced + (causal - forced) * (1.0 - std::pow(1.0 - hit, m->per_seed ? 1.0 : (double)m->n_seeds)));
+}
+
+// Key lists of up to this many bytes, if every causal pair were kept, are allocated at that size by the
+// one-call entry points, which then need not wait for the mask's pair count: their whole call is
+// queued at once. (One call of 12 / 2 heads at N = 3001: 107 us with the wait, 83 without.)
+constexpr int64_t kUnsizedBytes = 64 << 20;
+
+// ris_mask_generate; sized = false: if the key lists are small enough (kUnsizedBytes), nothing is read
+// back and n_pairs, which only chooses the design of a call, is the expected count.
+ris_status build_mask(int64_t N, int32_t kv_heads, int32_t mode, double density, const uint32_t *seeds,
                              int32_t n_seeds, const ris_mask_opts *opts, int32_t per_seed, ris_mask_t *out_mask,
-                             void *stream)
+                             void *stream, bool sized)
 {
     if (out_mask == nullptr) return fail(RIS_ERR_INVALID, "out_mask is NULL");
     *out_mask = nullptr;
@@ -550,11 +575,15 @@ ris_status ris_mask_generate(int64_t N, int32_t kv_heads, int32_t mode, double d
     RIS_CUDA(partials.alloc(sizeof(int64_t) * (size_t)scan_partials_count(n_rows), s));
     RIS_CUDA(launch_scan_inplace(mk->row_ptr + 1, n_rows, (int64_t *)partials.p, s));
 
-    int64_t total = 0;
-    RIS_CUDA(cudaMemcpyAsync(&total, mk->row_ptr + n_rows, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    RIS_CUDA(cudaStreamSynchronize(s));
-    mk->n_pairs = total;
-    RIS_CUDA(pool_alloc(&mk->col, (size_t)(total > 0 ? total : 1) * mk->col_bytes, s));
+    int64_t room = n_masks * (N * (N + 1) / 2);  // at most: every causal pair
+    if (!sized && room <= kUnsizedBytes / mk->col_bytes) {
+        mk->n_pairs = (int64_t)(expected_pairs(mk, o) + 0.5);
+    } else {
+        RIS_CUDA(cudaMemcpyAsync(&room, mk->row_ptr + n_rows, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        RIS_CUDA(cudaStreamSynchronize(s));
+        mk->n_pairs = room;
+    }
+    RIS_CUDA(pool_alloc(&mk->col, (size_t)(room > 0 ? room : 1) * mk->col_bytes, s));
 
     MaskFillArgs f{};
     f.single_row = -1;
@@ -570,6 +599,17 @@ ris_status ris_mask_generate(int64_t N, int32_t kv_heads, int32_t mode, double d
     guard.m = nullptr;
     *out_mask = mk;
     return RIS_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+ris_status ris_mask_generate(int64_t N, int32_t kv_heads, int32_t mode, double density, const uint32_t *seeds,
+                             int32_t n_seeds, const ris_mask_opts *opts, int32_t per_seed, ris_mask_t *out_mask,
+                             void *stream)
+{
+    return build_mask(N, kv_heads, mode, density, seeds, n_seeds, opts, per_seed, out_mask, stream, true);
 }
 
 ris_status ris_mask_info(ris_mask_t m, ris_mask_desc *out)
@@ -665,7 +705,20 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
     const bool tile8 = dtype == RIS_BF16 && head_dim == 128 && rotated &&
                        (tile || ((suffix || design == 0) && aligned32(v)));
     const bool q_pair = tile || suffix || tile8;  // queries as a 16-bit pair (else fp32)
-    Scratch qt, qtl, kt, ktl, po, pl, v16, vmax, bound;
+    // Three pool allocations at most, each carved up below (a pair of pool calls costs the host a few
+    // microseconds, and a short layer has little else to wait for): the rotated queries, the rotated
+    // keys, and the values' part: max |v| or the three bounds, fp16 values, the split's partial outputs.
+    Scratch q_mem, k_mem, v_mem;
+    auto room = [](size_t bytes) { return (bytes + 255) & ~size_t(255); };
+    const size_t nv = (size_t)N * kv_heads * head_dim, n_part = (size_t)N * heads;
+    void *q_hi = nullptr, *q_low = nullptr, *k_hi = nullptr, *k_low = nullptr, *v16 = nullptr;
+    float *bound = nullptr;
+    if (tile || suffix || tile8) {
+        const size_t part = suffix ? room(n_part * head_dim * sizeof(float)) + n_part * sizeof(float) : 0;
+        RIS_CUDA(v_mem.alloc(256 + room(nv * 2) + part, s));
+        bound = (float *)v_mem.p;
+        v16 = (char *)v_mem.p + 256;
+    }
     const void *qu = q, *ku = k, *kl = nullptr, *q_lo = nullptr;
     bool q_split = false;
     if (rotated) {
@@ -678,28 +731,24 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
         // rotated queries: fp32 (split into bf16 hi + lo by the gather kernels) or a 16-bit pair
         // (the fp8 scheme's operands, or a bf16 hi + lo pair); rotated keys in fp32, or for bf16
         // inputs a 16-bit pair
-        if (q_pair) {
-            RIS_CUDA(qt.alloc(nq * 2, s));
-            RIS_CUDA(qtl.alloc(nq * 2, s));
-        } else {
-            RIS_CUDA(qt.alloc(nq * sizeof(float), s));
-        }
-        RIS_CUDA(kt.alloc(nk * (dtype == RIS_BF16 ? 2 : 4), s));
-        if (dtype == RIS_BF16) RIS_CUDA(ktl.alloc(nk * 2, s));
-        if (tile8) {
-            // bounds, then the operands and the values as fp16: two launches
-            RIS_CUDA(bound.alloc(3 * sizeof(float), s));
-            RIS_CUDA(v16.alloc(nk * 2, s));
+        const size_t q_bytes = room(nq * (q_pair ? 2 : 4)), k_bytes = room(nk * (dtype == RIS_BF16 ? 2 : 4));
+        RIS_CUDA(q_mem.alloc((q_pair ? 2 : 1) * q_bytes, s));
+        RIS_CUDA(k_mem.alloc((dtype == RIS_BF16 ? 2 : 1) * k_bytes, s));
+        q_hi = q_mem.p;
+        if (q_pair) q_low = (char *)q_mem.p + q_bytes;
+        k_hi = k_mem.p;
+        if (dtype == RIS_BF16) k_low = (char *)k_mem.p + k_bytes;
+        if (tile8) {  // bounds, then the operands and the values as fp16: two launches
             Fp8PrepArgs pa{};
             pa.q = q;
             pa.k = k;
             pa.v = v;
-            pa.q_hi = qt.p;
-            pa.q_lo = qtl.p;
-            pa.k_hi = kt.p;
-            pa.k_lo = ktl.p;
-            pa.v16 = v16.p;
-            pa.bounds = (float *)bound.p;
+            pa.q_hi = q_hi;
+            pa.q_lo = q_low;
+            pa.k_hi = k_hi;
+            pa.k_lo = k_low;
+            pa.v16 = v16;
+            pa.bounds = bound;
             pa.N = N;
             pa.q_rows = q_rows;
             pa.q_first = q_first;
@@ -713,10 +762,10 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
             RopeQkArgs ra{};
             ra.q = q;
             ra.k = k;
-            ra.q_out = qt.p;
-            ra.q_lo = qtl.p;
-            ra.k_out = kt.p;
-            ra.k_lo = ktl.p;
+            ra.q_out = q_hi;
+            ra.q_lo = q_low;
+            ra.k_out = k_hi;
+            ra.k_lo = k_low;
             ra.N = N;
             ra.q_rows = q_rows;
             ra.q_first = q_first;
@@ -727,10 +776,10 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
             ra.mscale = (float)ms;
             RIS_CUDA(launch_rope_qk(ra, dtype, s));
         }
-        qu = back(qt.p, (size_t)heads * head_dim * (q_pair ? 2 : 4));
-        q_lo = back(qtl.p, (size_t)heads * head_dim * 2);
-        ku = kt.p;
-        kl = ktl.p;
+        qu = back(q_hi, (size_t)heads * head_dim * (q_pair ? 2 : 4));
+        q_lo = back(q_low, (size_t)heads * head_dim * 2);
+        ku = k_hi;
+        kl = k_low;
         q_split = (dtype == RIS_BF16);
     }
     if (qu == q) qu = back(q, (size_t)heads * head_dim * (dtype == RIS_BF16 ? 2 : 4));
@@ -761,26 +810,19 @@ ris_status run_attention(const ris_mask_s *m, const void *q, const void *k, cons
     a.q_first = q_first;
     a.q_rows = q_rows;
     a.n_tasks = (int64_t)a.n_sets * (row1 - row0) * kv_heads;
-    a.qk_bound = tile8 ? (const float *)bound.p : nullptr;
-    if (tile || suffix || tile8) {
+    a.qk_bound = tile8 ? bound : nullptr;
+    if (v16 != nullptr) {
         // the value products of the tile kernel and of the gather's fp8 form take the values as
         // fp16 (scaled into range), written above with the fp8 operands or here
-        if (!tile8) {
-            const size_t nv = (size_t)N * kv_heads * head_dim;
-            RIS_CUDA(v16.alloc(nv * 2, s));
-            RIS_CUDA(vmax.alloc(sizeof(float), s));
-            RIS_CUDA(launch_values_f16(v, (int64_t)nv, v16.p, (float *)vmax.p, s));
-        }
-        a.v16 = v16.p;
-        a.v_absmax = tile8 ? (const float *)bound.p + 2 : (const float *)vmax.p;
+        if (!tile8) RIS_CUDA(launch_values_f16(v, (int64_t)nv, v16, bound, s));
+        a.v16 = v16;
+        a.v_absmax = tile8 ? bound + 2 : bound;
     }
     if (suffix) {
-        RIS_CUDA(po.alloc((size_t)N * heads * head_dim * sizeof(float), s));
-        RIS_CUDA(pl.alloc((size_t)N * heads * sizeof(float), s));
         a.clique_B = suffix_block(m);
         a.window = m->window;
-        a.part_o = (float *)po.p;
-        a.part_lse = (float *)pl.p;
+        a.part_o = (float *)((char *)v16 + room(nv * 2));
+        a.part_lse = (float *)((char *)a.part_o + room(n_part * head_dim * sizeof(float)));
     }
     const auto ev = timer_pair();
     if (ev.first) RIS_CUDA(cudaEventRecord(ev.first, s));
@@ -808,7 +850,7 @@ ris_status fwd_common(const void *q, const void *k, const void *v, void *out, in
     RIS_TRY(check_seeds(seeds, n_seeds));
     RIS_TRY(check_opts(opts));
     ris_mask_t m = nullptr;
-    RIS_TRY(ris_mask_generate(N, kv_heads, mode, density, seeds, n_seeds, opts, per_seed, &m, stream));
+    RIS_TRY(build_mask(N, kv_heads, mode, density, seeds, n_seeds, opts, per_seed, &m, stream, false));
     const ris_status st = run_attention(m, q, k, v, out, heads, kv_heads, head_dim, dtype, out_dtype, rope, lse,
                                         reinterpret_cast<cudaStream_t>(stream));
     const std::string keep = t_err;
