@@ -60,12 +60,18 @@
 //                         masking per tile more) is as slow as the pipe. There the groups' warps of a
 //                         scheduler ran their exponentials against each other, and a warp in a
 //                         hundred rescaled O, while seven others waited: the reference maximum is now
-//                         handed over after the exponentials, and moves at 2^14 instead of 2^8.
+//                         handed over after the exponentials, and moves at 2^14 instead of 2^8;
+//   1,590 / 1,850         row sums that add fp16 as it is, -infinity by predicated moves, the next
+//                         tile's scores polled for ahead of their use.
 // A CTA's start and end, 16,000 cycles with the query rows loaded and the output rows stored 16 bytes
 // per lane and row, take 7,000 with the query tile loaded by TMA and the output through
 // shared memory.
-// Layer calls, before -> now: N = 8192 306 -> 248 us, 32k dense 3.77 -> 2.98 ms, 64k 14.1 -> 11.5 ms.
-// Not kept: more polls between two reads of the error word in a wait (3% slower at N = 8192), a
+// Layer calls, before -> now: N = 8192 306 -> 225 us (23 of them in other kernels), 32k dense
+// 3.77 -> 2.89 ms, 64k 14.1 -> 11.2 ms.
+// Not kept: the bitmap applied to P as packed masks, with the maximum taken over all keys and again
+// over the kept ones only where it could move (fewer instructions, but in the exponentials' chain
+// from group to group: N = 8192 226 -> 244 us), the first loads ahead of the TMEM allocation
+// (231 -> 234), more polls between two reads of the error word in a wait (3% slower at N = 8192), a
 // suspend-time hint on the polls (no change).
 //
 // The suffix pass of the dense-suffix split (SUFFIX) runs the same pipeline over the key
@@ -224,6 +230,19 @@ __device__ __forceinline__ bool mbar_wait_own(uint32_t bar, uint32_t parity)
     while (!mbar_try_wait(bar, parity))
         if (clock64() - t0 > (1LL << 31)) return false;
     return true;
+}
+
+// Whether the phase has completed by now: asked ahead of the wait, so that a completed one costs
+// no round trip to the barrier at the point of use
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
 }
 
 // Bounded wait (`limit` cycles, about 2^31 unless a test lowers it); false if the phase did
@@ -488,8 +507,26 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
-// Two fp32 values in one 64-bit register, and their packed fused multiply-add and sum (each
-// half rounded as the scalar operation).
+// a + b of an fp16 b, both exact operands of one fp32 addition
+__device__ __forceinline__ float add_f16(float a, __half b)
+{
+    float r;
+    asm("add.rn.f32.f16 %0, %1, %2;" : "=f"(r) : "h"(__half_as_ushort(b)), "f"(a));
+    return r;
+}
+
+// x = -infinity unless the word has the bit: a predicated move, which unlike a selection of two
+// registers need not run on the integer pipe that the test is on
+__device__ __forceinline__ void drop_unless(float &x, uint32_t word, uint32_t bit)
+{
+    asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+        "and.b32 t, %1, %2;\n\tsetp.eq.u32 p, t, 0;\n\t@p mov.b32 %0, 0xFF800000;\n\t}"
+        : "+f"(x)
+        : "r"(word), "r"(bit));
+}
+
+// Two fp32 values in one 64-bit register, and their packed fused multiply-add (each half
+// rounded as the scalar operation).
 __device__ __forceinline__ uint64_t f2_pack(float x, float y)
 {
     uint64_t d;
@@ -504,12 +541,6 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c)
 {
     uint64_t d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 
@@ -880,9 +911,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         const uint64_t sc2 = f2_pack(sc, sc);
         float l = 0.f, m_own = -INFINITY;  // row sum over this thread's tiles, relative to 2^m_own
+        bool s_full = false;  // seen at the end of the last tile: a poll takes 200 cycles even if it succeeds
         for (int j = grp; j < n_kt; j += 2) {
             if (!kRange) mask_words(j + 4, nnw);
-            if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1, wl));
+            if (ok) ok = __all_sync(0xFFFFFFFFu, s_full || mbar_wait(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1, wl));
             tc_fence_after();
             uint32_t su[2][64];
             tmem_issue64(T_S0 + grp * BN + lane_off, su[0]);
@@ -903,7 +935,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int c = 0; c < BN; ++c) sv[c] = __uint_as_float(su[c >> 6][c & 63]);
             if (!whole) {
 #pragma unroll
-                for (int c = 0; c < BN; ++c) sv[c] = ((cw[c >> 5] >> (c & 31)) & 1u) ? sv[c] : -INFINITY;
+                for (int c = 0; c < BN; ++c) drop_unless(sv[c], cw[c >> 5], 1u << (c & 31));
             }
             if (!kRange) {
 #pragma unroll
@@ -964,8 +996,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             // P = exp2(s - m_ref) as the A operand of the value product, packed two keys per
             // column. The row sum adds P as rounded, so that the rounding of each weight moves the
             // output by at most 2^-11 of the weight times |v_j - o| (a normalised average of the
-            // values with slightly perturbed weights).
-            uint64_t lsum[2] = {0ull, 0ull};
+            // values with slightly perturbed weights). The additions take the fp16 halves as they are:
+            // this loop alone, two warps of a scheduler, 690 cycles a tile with conversions and packed
+            // additions, 600 so, 540 for the exponentials and their arguments only.
+            float lsum[4] = {};
             const uint64_t nmu2 = f2_pack(-mu, -mu);
             uint32_t hw[BN / 2];
 #pragma unroll
@@ -973,8 +1007,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float x0, x1;
                 f2_unpack(f2_fma(f2_pack(sv[2 * w], sv[2 * w + 1]), sc2, nmu2), x0, x1);
                 const __half2 hp = __floats2half2_rn(ex2(x0), ex2(x1));
-                const float2 pr = __half22float2(hp);
-                lsum[w & 1] = f2_add(lsum[w & 1], f2_pack(pr.x, pr.y));
+                lsum[2 * (w & 1)] = add_f16(lsum[2 * (w & 1)], __low2half(hp));
+                lsum[2 * (w & 1) + 1] = add_f16(lsum[2 * (w & 1) + 1], __high2half(hp));
                 hw[w] = *reinterpret_cast<const uint32_t *>(&hp);
             }
             // Only now on to the other group: its exponentials (the other warp of this scheduler) run
@@ -992,9 +1026,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t tp = T_P0 + grp * (BN / 2) + lane_off;
             tmem_st32(tp, hw);
             tmem_st32(tp + 32, hw + 32);
-            float la, lb;
-            f2_unpack(f2_add(lsum[0], lsum[1]), la, lb);
-            l += la + lb;
+            s_full = j + 2 < n_kt && mbar_test(sbase + BAR(L::B_S_FULL + (j + 2) % NSK), ((j + 2) / NSK) & 1);
+            l += (lsum[0] + lsum[2]) + (lsum[1] + lsum[3]);
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
