@@ -255,7 +255,7 @@ __device__ __forceinline__ int velem(int j, int p)
     return (WIDE && D == 128) ? 16 * p + 2 * j : 64 * (j >> 2) + 8 * p + 2 * (j & 3);
 }
 
-constexpr float kLazyLog2 = 14.f;  // rescale O only when the row maximum grows by more than 2^14 (P in fp16's range)
+constexpr float kLazyLog2 = 8.f;  // rescale O only when the row maximum grows by more than 2^8
 
 // D: head dim (64 or 128). QSPLIT: q is fp32 (split hi + lo); else q is bf16.
 // KSPLIT: keys come as a bf16 hi (a.k) + lo (a.k_lo) pair. WIDE: 32-byte loads (K, K lo and

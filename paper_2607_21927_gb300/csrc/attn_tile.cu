@@ -24,7 +24,7 @@
 //                   tiles: per tile tcgen05.ld the row's 128 scores, apply the bitmap (words
 //                   fetched four tiles ahead) or the causal cut, take the row max, fp32 online
 //                   softmax from the reference maximum that the other group hands over, with lazy
-//                   rescaling of O in TMEM (only when the row max grows by more than 2^14), write P
+//                   rescaling of O in TMEM (only when the row max grows by more than 2^8), write P
 //                   into TMEM, and at the end normalise O (and undo the values' power-of-two
 //                   scale) and store it, coalesced, through shared memory.
 //
@@ -60,14 +60,16 @@
 //                         masking per tile more) is as slow as the pipe. There the groups' warps of a
 //                         scheduler ran their exponentials against each other, and a warp in a
 //                         hundred rescaled O, while seven others waited: the reference maximum is now
-//                         handed over after the exponentials, and moves at 2^14 instead of 2^8;
-//   1,590 / 1,850         row sums that add fp16 as it is, -infinity by predicated moves, the next
+//                         handed over after the exponentials (it still moves at 2^8: 2^14 gains 2% at
+//                         N = 8192 and 1% at 64k, but then the heaviest weight of a row is less
+//                         often exactly 1, and the log-sum-exp of a dense 32k layer is 5% further off);
+//   1,650 / 1,870         row sums that add fp16 as it is, -infinity by predicated moves, the next
 //                         tile's scores polled for ahead of their use.
 // A CTA's start and end, 16,000 cycles with the query rows loaded and the output rows stored 16 bytes
 // per lane and row, take 7,000 with the query tile loaded by TMA and the output through
 // shared memory.
-// Layer calls, before -> now: N = 8192 306 -> 225 us (23 of them in other kernels), 32k dense
-// 3.77 -> 2.89 ms, 64k 14.1 -> 11.2 ms.
+// Layer calls, before -> now: N = 8192 306 -> 229 us, 32k dense 3.74 -> 2.90 ms, 64k
+// 14.0 -> 11.3 ms.
 // Not kept: the bitmap applied to P as packed masks, with the maximum taken over all keys and again
 // over the kept ones only where it could move (fewer instructions, but in the exponentials' chain
 // from group to group: N = 8192 226 -> 244 us), the first loads ahead of the TMEM allocation
@@ -115,11 +117,9 @@ constexpr int kThreads = 32 * (kSoftmaxWarps + 4);
 // registers per thread: at launch, then after setmaxnreg of a softmax and of a loader / MMA thread
 constexpr int kRegs = 168, kSoftmaxRegs = 200, kOtherRegs = 104;
 static_assert(2 * kSoftmaxRegs + kOtherRegs == 3 * kRegs, "the shares of the three warpgroups add up to the launch's");
-// The reference maximum of a row moves only when its maximum grows by more than this (log2): P
-// stays below 2^14, inside fp16, and a lower reference only keeps more of the small weights out of
-// fp16's subnormals. On a 10% mask of 64k tokens one warp in a hundred rescaled O in a tile at a
-// step of 2^8, and a tile waits for the slowest of eight warps.
-constexpr float kLazyLog2 = 14.f;
+// The reference maximum of a row moves only when its maximum grows by more than this (log2), so P
+// stays below 2^8. On a 10% mask of 64k tokens one warp in a hundred rescales O in a tile.
+constexpr float kLazyLog2 = 8.f;
 constexpr uint32_t kTmemCols = 512;  // S (2 x 128) + O (128) + P (2 x 64)
 
 // How the kernel of head dim DT (128 or 64) is laid out. At 128 two CTAs of a cluster share their
