@@ -64,7 +64,7 @@ struct RowDraws {
 // 4 g .. 4 g + 4 U - 1): a key is kept by some seed iff this minimum is below the threshold.
 //
 // Philox4x32-10 as in philox4x32_10 above, with what the 10 rounds of a row's calls have in common
-// taken out of the loop over seeds. Round 1 multiplies the group (word 0) and the stream (word 2),
+// taken out of the loop over seeds (SEEDS a pass; 0: one seed in all, s0, without a loop or minima). Round 1 multiplies the group (word 0) and the stream (word 2),
 // neither of which depends on the seed; its results z, w depend on the group only (key word 1 is
 // the head key) and x, y on the row and seed only. So the second product of round 2 depends on the
 // group only and the first on the seed only: per call 8 rounds of two products remain, 16 of 20.
@@ -83,8 +83,9 @@ __device__ __forceinline__ void min_words(const MaskBitsArgs &a, const RowDraws 
 #pragma unroll
         for (int e = 0; e < 4; ++e) best[u][e] = 0xFFFFFFFFu;
     }
-#pragma unroll SEEDS
-    for (int s = s0; s < s1; ++s) {
+    const int end = SEEDS == 0 ? s0 + 1 : s1;
+#pragma unroll(SEEDS == 0 ? 1 : SEEDS)
+    for (int s = s0; s < end; ++s) {
         uint32_t k0 = a.seeds.v[s], k1 = d.k1 + 0xBB67AE85u;
         const uint64_t ps = (uint64_t)0xD2511F53u * (d.s_hi ^ d.i ^ k0);
         k0 += 0x9E3779B9u;
@@ -114,75 +115,126 @@ __device__ __forceinline__ void min_words(const MaskBitsArgs &a, const RowDraws 
     }
 }
 
-// One CTA per (mask, row), one warp per 16 words (512 keys) at a time: lane l takes the 16 keys of
-// half a word, groups 4 l .. 4 l + 3 of the step's 128, and its neighbour the other half.
+// A (mask, row) of the launch: its bitmap row, its words and drawn groups, its forced keys.
+struct RowTask {
+    uint32_t *row;
+    int i, nw, ng, tail0, last;
+    int s0, s1;    // its seeds
+    uint32_t tm1;  // u < thr for thr in [1, 2^32] is u <= thr - 1 in 32 bits
+    RowDraws d;
+};
+
+__device__ __forceinline__ RowTask row_task(const MaskBitsArgs &a, uint32_t m, int i)
+{
+    const bool one = a.single_row >= 0;
+    RowTask t;
+    t.i = i;
+    t.s0 = a.per_seed ? (int)m / a.heads_keyed : 0;
+    t.s1 = a.per_seed ? t.s0 + 1 : a.n_seeds;
+    t.row = a.bitmap + (int64_t)m * a.words_per_mask + (one ? 0 : row_word_offset(i));
+    // forced keys: local window (i-W, i], anchors [0, A), Structural clique [block start, i]; the draws
+    // matter for j < i before the first and the last
+    t.tail0 = i - a.W + 1;
+    if (a.mode == RIS_MODE_STRUCTURAL) t.tail0 = min(t.tail0, (int)((uint32_t)i / (uint32_t)a.B * (uint32_t)a.B));
+    t.last = one ? i - 1 : i;  // a single row keeps keys j < i only
+    t.nw = (i >> 5) + 1;
+    t.ng = a.thr > 0 ? (max(0, min(i, t.tail0)) + 3) >> 2 : 0;
+    t.tm1 = a.thr > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)(a.thr - 1);
+    t.d.i = (uint32_t)i;
+    t.d.layer = a.layer_key;
+    t.d.k1 = (a.heads_keyed > 1) ? m % (uint32_t)a.heads_keyed : 0u;
+    const uint64_t ps = (uint64_t)0xCD9E8D57u * a.stream;
+    t.d.s_hi = (uint32_t)(ps >> 32);
+    t.d.s_lo = (uint32_t)ps;
+    return t;
+}
+
+// One warp, 16 words (512 keys) from word w0 on: lane l takes the 16 keys of half a word, groups
+// 4 l .. 4 l + 3 of the step's 128, and its neighbour the other half. Returns the lane's kept keys.
+template <int SEEDS>
+__device__ __forceinline__ int row_step(const MaskBitsArgs &a, const RowTask &t, int w0, int lane)
+{
+    uint32_t word = 0u;
+    if (8 * w0 < t.ng) {
+        uint32_t best[4][4];
+        min_words<4, SEEDS>(a, t.d, (uint32_t)(8 * w0 + 4 * lane), t.s0, t.s1, best);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) word |= best[e >> 2][e & 3] <= t.tm1 ? 1u << e : 0u;
+    }
+    word |= __shfl_down_sync(0xFFFFFFFFu, word, 1) << 16;
+    const int w = w0 + (lane >> 1);
+    if ((lane & 1) != 0 || w >= t.nw) return 0;
+    const int j0 = w << 5;
+    uint32_t bits = word & bits_to(t.i - 1 - j0);  // drawn pairs are j < i
+    if (a.or_existing) bits |= t.row[w];
+    bits = (bits | bits_from(t.tail0 - j0) | bits_to(a.A - 1 - j0)) & bits_to(t.last - j0);
+    t.row[w] = bits;
+    return __popc(bits);
+}
+
+// One CTA per (mask, row), rows from the last (longest) to the first, its warps 16 words apart.
 //
 // Bound by the 32 x 32 -> 64-bit products (32 lanes per clock and SM, a quarter of the fp32 rate)
 // and, nearly as much, by the ALU pipe (an exclusive or per product, the minima, the key schedule).
-// MANY: two seeds per loop pass and as many registers as the compiler wants (the key schedules stay in
-// registers); else eight CTAs per SM, for masks of one or two seeds, where a row's other work
-// counts. Measured at N = 16384 of 1% (few / many): 1 seed 138 / 144 us, 2 217 / 217, 3 297 / 283, 8 693 /
-// 641, 20 1644 / 1487. 70 seeds at N = 32768: 29.0 ms with every round in the loop over seeds and one
-// thread per word, 21.1 with rounds 1 and 2 taken out, 19.6 now (1.5 calls per clock and SM).
-constexpr int kManySeeds = 3;
-template <bool MANY>
-__global__ void __launch_bounds__(kBitsThreads, MANY ? 1 : 8) k_mask_bits(const MaskBitsArgs a)
+// SEEDS = 2: as many registers as the compiler wants (the key schedules stay in registers). Measured at N =
+// 16384 of 1% (one seed per pass and eight CTAs per SM / two per pass): 2 seeds 217 / 209 us, 3 297 / 283,
+// 8 693 / 641, 20 1644 / 1487. 70 seeds at N = 32768: 29.0 ms with every round in the loop over seeds and one thread
+// per word, 21.1 with rounds 1 and 2 taken out, 19.6 now (1.5 calls per clock and SM). SEEDS = 0, one seed: eight
+// CTAs per SM, a row's other work counts.
+template <int SEEDS>
+__global__ void __launch_bounds__(kBitsThreads, SEEDS > 0 ? 1 : 8) k_mask_bits(const MaskBitsArgs a)
 {
-    // rows are visited from the last (longest) to the first
     const uint32_t m = blockIdx.x % (uint32_t)a.n_masks;
     const bool one = a.single_row >= 0;
     const int i = (int)(one ? a.single_row : a.N - 1 - blockIdx.x / (uint32_t)a.n_masks);  // below 2^31
-    const int32_t s0 = a.per_seed ? (int)m / a.heads_keyed : 0;
-    const int32_t s1 = a.per_seed ? s0 + 1 : a.n_seeds;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *row = a.bitmap + (int64_t)m * a.words_per_mask + (one ? 0 : row_word_offset(i));
-    // forced keys: local window (i-W, i], anchors [0, A), Structural clique [block start, i]; the draws
-    // matter for j < i before the first and the last
-    int tail0 = i - a.W + 1;
-    if (a.mode == RIS_MODE_STRUCTURAL) tail0 = min(tail0, (int)((uint32_t)i / (uint32_t)a.B * (uint32_t)a.B));
-    const int last = one ? i - 1 : i;  // a single row keeps keys j < i only
-    const int nw = (i >> 5) + 1;
-    const int ng = a.thr > 0 ? (max(0, min(i, tail0)) + 3) >> 2 : 0;
-    // u < thr for thr in [1, 2^32] is u <= thr - 1 in 32 bits
-    const uint32_t tm1 = a.thr > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)(a.thr - 1);
-    RowDraws d;
-    d.i = (uint32_t)i;
-    d.layer = a.layer_key;
-    d.k1 = (a.heads_keyed > 1) ? m % (uint32_t)a.heads_keyed : 0u;
-    const uint64_t ps = (uint64_t)0xCD9E8D57u * a.stream;
-    d.s_hi = (uint32_t)(ps >> 32);
-    d.s_lo = (uint32_t)ps;
-
+    const RowTask t = row_task(a, m, i);
     int count = 0;
-    for (int w0 = 16 * warp; w0 < nw; w0 += 16 * (kBitsThreads / 32)) {
-        uint32_t word = 0u;
-        if (8 * w0 < ng) {
-            uint32_t best[4][4];
-            min_words<4, MANY ? 2 : 1>(a, d, (uint32_t)(8 * w0 + 4 * lane), s0, s1, best);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) word |= best[e >> 2][e & 3] <= tm1 ? 1u << e : 0u;
-        }
-        word |= __shfl_down_sync(0xFFFFFFFFu, word, 1) << 16;
-        const int w = w0 + (lane >> 1);
-        if ((lane & 1) == 0 && w < nw) {
-            const int j0 = w << 5;
-            uint32_t bits = word & bits_to(i - 1 - j0);  // drawn pairs are j < i
-            if (a.or_existing) bits |= row[w];
-            bits = (bits | bits_from(tail0 - j0) | bits_to(a.A - 1 - j0)) & bits_to(last - j0);
-            row[w] = bits;
-            count += __popc(bits);
-        }
-    }
+    for (int w0 = 16 * warp; w0 < t.nw; w0 += 16 * (kBitsThreads / 32)) count += row_step<SEEDS>(a, t, w0, lane);
     // block reduction of the row count
     __shared__ int red[kBitsThreads / 32];
     count = __reduce_add_sync(0xFFFFFFFFu, count);
     if (lane == 0) red[warp] = count;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int t = 0;  // a row holds at most 2^31 - 1 keys
+        int n = 0;  // a row holds at most 2^31 - 1 keys
 #pragma unroll
-        for (int k = 0; k < kBitsThreads / 32; ++k) t += red[k];
-        a.counts[one ? (int64_t)m : (int64_t)m * a.N + i] = t;
+        for (int k = 0; k < kBitsThreads / 32; ++k) n += red[k];
+        a.counts[one ? (int64_t)m : (int64_t)m * a.N + i] = n;
+    }
+}
+
+// One seed per mask and rows enough for four of them per CTA (the caller sees to both): the steps of
+// the four rows one after the other, dealt to the warps in turn. With one call per four keys a CTA's
+// start, its last step and its end are a good part of a short row: ten one-seed masks of N = 8192 take 345 us
+// against 360 with one row per CTA (367 with the loop over seeds and its minima), one of N = 16384 121-127
+// against 130 (138).
+constexpr int kOneSeedRows = 4;
+__global__ void __launch_bounds__(kBitsThreads, 6) k_mask_bits_one(const MaskBitsArgs a)
+{
+    const uint32_t tasks = (uint32_t)(a.N * a.n_masks), t0 = blockIdx.x * (uint32_t)kOneSeedRows;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ int total[kOneSeedRows];
+    if (threadIdx.x < kOneSeedRows) total[threadIdx.x] = 0;
+    __syncthreads();
+    int at = warp;  // the warp's next step, from the start of row q
+#pragma unroll 1
+    for (int q = 0; q < kOneSeedRows && t0 + q < tasks; ++q) {
+        const uint32_t r = (t0 + q) / (uint32_t)a.n_masks, m = t0 + q - r * (uint32_t)a.n_masks;
+        const int i = (int)(a.N - 1 - r), steps = ((i >> 5) + 16) >> 4;
+        if (at < steps) {
+            const RowTask t = row_task(a, m, i);
+            int count = 0;
+            for (; at < steps; at += kBitsThreads / 32) count += row_step<0>(a, t, 16 * at, lane);
+            count = __reduce_add_sync(0xFFFFFFFFu, count);
+            if (lane == 0) atomicAdd(&total[q], count);
+        }
+        at -= steps;
+    }
+    __syncthreads();
+    if (threadIdx.x < kOneSeedRows && t0 + threadIdx.x < tasks) {
+        const uint32_t t = t0 + threadIdx.x, r = t / (uint32_t)a.n_masks;
+        a.counts[(int64_t)(t - r * (uint32_t)a.n_masks) * a.N + (a.N - 1 - r)] = total[threadIdx.x];
     }
 }
 
@@ -370,10 +422,15 @@ __global__ void __launch_bounds__(kFillThreads) k_mask_fill(const MaskFillArgs a
 cudaError_t launch_mask_bits(const MaskBitsArgs &a, cudaStream_t s)
 {
     const int64_t blocks = (int64_t)a.n_masks * (a.single_row >= 0 ? 1 : a.N);
-    if ((a.per_seed ? 1 : a.n_seeds) >= kManySeeds)
-        k_mask_bits<true><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
+    const int seeds = a.per_seed ? 1 : a.n_seeds;
+    // four rows per CTA only if that leaves sixteen CTAs per SM: below, rows in flight count for more
+    // (N = 2048, one seed: 7.3 us against 6.4)
+    if (seeds == 1 && a.single_row < 0 && blocks >= (int64_t)kOneSeedRows * 16 * 152)
+        k_mask_bits_one<<<(unsigned)((blocks + kOneSeedRows - 1) / kOneSeedRows), kBitsThreads, 0, s>>>(a);
+    else if (seeds == 1)
+        k_mask_bits<0><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
     else
-        k_mask_bits<false><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
+        k_mask_bits<2><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
     note_launch();
     return cudaGetLastError();
 }

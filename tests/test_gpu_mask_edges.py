@@ -1,5 +1,5 @@
 """Mask sampler at the edges of its steps: rows around one word and around a warp's 512 keys, odd and
-even seed counts on both sides of the few / many line, windows and anchors at their extremes."""
+even seed counts, one seed and more, windows and anchors at their extremes."""
 import numpy as np
 import pytest
 
@@ -22,3 +22,14 @@ def test_mask_steps(N, S, mode, W, A, head_keyed, sampler):
              for h in heads]
     rows = np.unique(np.clip([0, 1, 30, 31, 32, 510, 511, 512, 513, 2047, 2048, 2049, N - 2, N - 1], 0, N - 1))
     check_rows(m, specs, rows)
+
+
+@pytest.mark.parametrize("N,heads,mode,W,A", [
+    (2430, 4, 0, 1, 0),     # 9720 rows: one below the line of four rows per block
+    (2433, 4, 0, 1, 0),     # 9732: just above it
+    (2050, 5, 1, 700, 33),  # 10250: the last block has two rows
+    (9729, 1, 0, 1, 0)])
+def test_one_seed_rows(N, heads, mode, W, A):
+    m = gpu_mask(N, mode, 0.03, [77], kv_heads=heads, W=W, A=A, per_head=heads > 1, layer_key=5)
+    specs = [oracle_spec(N, mode, 0.03, [77], W=W, A=A, head_key=h, layer_key=5) for h in range(heads)]
+    check_rows(m, specs, np.unique([0, 1, 2, 3, 4, 31, 511, 512, 513, 2047, 2048, N - 3, N - 2, N - 1]))
