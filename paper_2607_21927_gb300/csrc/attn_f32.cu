@@ -17,7 +17,8 @@
 // heads in a group (layer call of one head at N = 2048: 31.4 against 33.3 us; six heads at N = 6007:
 // 291 us with three, 314 with two, 401 with four, which spill).
 // Layer calls, before (one lane per key row, 32 lines per load, groups padded to eight heads) -> now:
-// 12 / 2 heads of 128, N = 6007, 4.9% of the pairs: 492 -> 291 us; one head, N = 2048, 5%: 51 -> 31 us.
+// 12 / 2 heads of 128, N = 6007, 4.9% of the pairs: 492 -> 274 us; one head, N = 2048, 5%: 50 -> 28 us (17 and 3 us of them by the
+// launch that rotates q and k together and the shorter host path).
 #include <cuda_bf16.h>
 
 #include <cstdint>

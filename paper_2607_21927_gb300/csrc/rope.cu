@@ -1,11 +1,12 @@
 // RoPE with position extension (paper, Methods, "Dynamic RoPE Scaling"; linear and YaRN
 // per Results, "RoPE Scaling: Linear versus YaRN"; YaRN per Peng et al. 2023).
 //
-// One thread per (token p, frequency c) rotates the pair (c, c + D/2) of every head of the
+// k_rope: one thread per (token p, frequency c) rotates the pair (c, c + D/2) of every head of the
 // token: the angle p * f_c is formed in fp64 and reduced to [-pi, pi] in fp64 (an fp32
 // product loses ~4e-3 rad at p = 65535), then sin/cos of the reduced angle come from the
 // CUDA math library in fp32 and the rotation runs in fp32. The work is HBM-bound: one read
-// and one write of the tensor. For the fp16 + e4m3 score operands (head dim 128, bf16 inputs)
+// and one write of the tensor. A layer call rotates q and k in one launch (k_rope_qk) with 16-byte
+// accesses and the angle as a 64-bit fixed-point fraction of a turn. For the fp16 + e4m3 score operands (head dim 128, bf16 inputs)
 // two launches serve a whole layer call: k_fp8_bounds bounds q, k (and v) in one pass, then
 // k_fp8_rotate rotates q and k (one thread per token and 8 frequencies, 16-byte accesses) into
 // those operands and writes the fp16 values.
