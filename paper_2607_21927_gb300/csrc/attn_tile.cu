@@ -60,16 +60,17 @@
 //                         masking per tile more) is as slow as the pipe. There the groups' warps of a
 //                         scheduler ran their exponentials against each other, and a warp in a
 //                         hundred rescaled O, while seven others waited: the reference maximum is now
-//                         handed over after the exponentials (it still moves at 2^8: 2^14 gains 2% at
-//                         N = 8192 and 1% at 64k, but then the heaviest weight of a row is less
-//                         often exactly 1, and the log-sum-exp of a dense 32k layer is 5% further off);
+//                         handed over after the exponentials (it still moves at 2^8: at 2^14 the heaviest
+//                         weight of a row is less often exactly 1, and the log-sum-exp of a dense
+//                         32k layer is 5% further off);
 //   1,650 / 1,870         row sums that add fp16 as it is, -infinity by predicated moves, the next
-//                         tile's scores polled for ahead of their use.
+//                         tile's scores polled for ahead of their use. Then O is rescaled after the
+//                         exponentials and the hand-over instead of before: N = 8192 230 -> 226 us.
 // A CTA's start and end, 16,000 cycles with the query rows loaded and the output rows stored 16 bytes
 // per lane and row, take 7,000 with the query tile loaded by TMA and the output through
 // shared memory.
-// Layer calls, before -> now: N = 8192 306 -> 229 us, 32k dense 3.74 -> 2.90 ms, 64k
-// 14.0 -> 11.3 ms.
+// Layer calls, before -> now: N = 8192 306 -> 226 us, 32k dense 3.75 -> 2.90 ms, 64k
+// 14.0 -> 11.2 ms.
 // Not kept: the bitmap applied to P as packed masks, with the maximum taken over all keys and again
 // over the kept ones only where it could move (fewer instructions, but in the exponentials' chain
 // from group to group: N = 8192 226 -> 244 us), the first loads ahead of the TMEM allocation
@@ -971,23 +972,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 return t < 0 || __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
             };
             const bool scale_o = upd && m_prev != -INFINITY;
-            if (ok && __any_sync(0xFFFFFFFFu, scale_o)) {
-                // O has settled once the value product of tile j - 1 is done; that of tile j - 2 first, so
-                // that the barrier is not polled a phase early
-                ok = pv_done(j - 2) && pv_done(j - 1);
-                tc_fence_after();
-                const float al = scale_o ? exp2f(m_prev - m_ref) : 1.f;
-#pragma unroll 1
-                for (int c0 = 0; c0 < DT && ok; c0 += 32) {
-                    float ov[32];
-                    uint32_t ow[32];
-                    tmem_ld32(T_O + lane_off + c0, ov);
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) ow[c] = __float_as_uint(ov[c] * al);
-                    tmem_st32(T_O + lane_off + c0, ow);
-                }
-                tmem_wait_st();
-            }
+            const bool any_scale = __any_sync(0xFFFFFFFFu, scale_o);
+            const float al = scale_o ? exp2f(m_prev - m_ref) : 1.f;
             if (m_ref != m_own) {
                 l *= m_own == -INFINITY ? 0.f : exp2f(m_own - m_ref);
                 m_own = m_ref;
@@ -1023,6 +1009,25 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = pv_done(j - 2);  // P's buffer is free
             if (!ok) continue;
             tc_fence_after();
+            if (any_scale) {
+                // O has settled once the value product of tile j - 1 is done (that of tile j - 2 first, above, so
+                // that the barrier is not polled a phase early); nothing adds to it before this warp's
+                // P is announced below, and the other group's warp of these rows scales it next only after that product.
+                // Here and not ahead of the exponentials, where the wait held up the other group as well.
+                ok = pv_done(j - 1);
+                if (!ok) continue;
+                tc_fence_after();
+#pragma unroll 1
+                for (int c0 = 0; c0 < DT; c0 += 32) {
+                    float ov[32];
+                    uint32_t ow[32];
+                    tmem_ld32(T_O + lane_off + c0, ov);
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) ow[c] = __float_as_uint(ov[c] * al);
+                    tmem_st32(T_O + lane_off + c0, ow);
+                }
+                tmem_wait_st();
+            }
             const uint32_t tp = T_P0 + grp * (BN / 2) + lane_off;
             tmem_st32(tp, hw);
             tmem_st32(tp + 32, hw + 32);
