@@ -68,14 +68,14 @@
 //                         exponentials and the hand-over instead of before: N = 8192 230 -> 226 us.
 // A CTA's start and end, 16,000 cycles with the query rows loaded and the output rows stored 16 bytes
 // per lane and row, take 7,000 with the query tile loaded by TMA and the output through
-// shared memory.
-// Layer calls, before -> now: N = 8192 306 -> 226 us, 32k dense 3.75 -> 2.90 ms, 64k
-// 14.0 -> 11.2 ms.
+// shared memory; the first loads ahead of the TMEM allocation and the cluster barrier then took N =
+// 8192 from 224 to 221 us.
+// Layer calls, before -> now: N = 8192 306 -> 222 us, 32k dense 3.75 -> 2.90 ms, 64k
+// 14.0 -> 11.1 ms.
 // Not kept: the bitmap applied to P as packed masks, with the maximum taken over all keys and again
 // over the kept ones only where it could move (fewer instructions, but in the exponentials' chain
-// from group to group: N = 8192 226 -> 244 us), the first loads ahead of the TMEM allocation
-// (231 -> 234), more polls between two reads of the error word in a wait (3% slower at N = 8192), a
-// suspend-time hint on the polls (no change).
+// from group to group: N = 8192 226 -> 244 us), more polls between two reads of the error word in a
+// wait (3% slower at N = 8192), a suspend-time hint on the polls (no change).
 //
 // The suffix pass of the dense-suffix split (SUFFIX) runs the same pipeline over the key
 // tiles of each row's dense suffix only (its Structural block and / or local window: every key
@@ -638,15 +638,31 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int kt0 = SUFFIX ? (int)(dense_suffix_start(a, (int64_t)max(qt_lo, qt_first) * BM) / BN) : 0;
     const int n_kt = (int)(last_row / BN) + 1 - kt0;
 
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < L::NBAR; ++i) {
-            uint32_t cnt = 1;
-            // the group's warps and the relay, of each CTA
-            if ((i >= L::B_S_GO && i < L::B_S_GO + NSK) || (i >= L::B_P_GO && i < L::B_P_GO + NSV)) cnt = (kGroupWarps + 1) * CG;
-            mbar_init(smem_u32(&bars[i]), cnt);
+    const bool first_loads = a.debug_no_loads == 0 && (sbase & 1023u) == 0u;
+    if (warp == kTmaWarp) {
+        static_assert(L::NBAR <= 32, "a lane per barrier");
+        if (lane < L::NBAR) {
+            // S_GO, P_GO: the group's warps and the relay, of each CTA
+            const bool go = (lane >= L::B_S_GO && lane < L::B_S_GO + NSK) || (lane >= L::B_P_GO && lane < L::B_P_GO + NSV);
+            mbar_init(smem_u32(&bars[lane]), go ? (kGroupWarps + 1) * CG : 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        // the query tile and the first keys at once, under the rest of the start-up (about 2,000 cycles
+        // of TMEM allocation and cluster barrier): only this CTA's own barriers are involved
+        if (lane == 0 && first_loads) {
+            const uint32_t bq = sbase + L::OFF_BARS + 8 * L::B_Q_FULL, bk = sbase + L::OFF_BARS + 8 * L::B_K_FULL;
+            const int key = kt0 * BN + L::KROWS * rank;
+            mbar_arrive_expect_tx(bq, (SPLIT ? 2 : 1) * L::Q_ARR);
+            mbar_arrive_expect_tx(bk, (SPLIT ? 2 : 1) * L::K_ARR);
+            for (int blk = 0; blk < NB; ++blk) {
+                tma_load_3d(sbase + L::OFF_Q + blk * L::Q_BLK, &maps.qh, 64 * blk, h, (int)(q0 - a.q_first), bq);
+                if (SPLIT) tma_load_3d(sbase + L::OFF_Q + L::Q_ARR + blk * L::Q_BLK, &maps.ql, 64 * blk, h, (int)(q0 - a.q_first), bq);
+                tma_load_3d(sbase + L::OFF_K + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
+                if (SPLIT) tma_load_3d(sbase + L::OFF_K + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
+            }
+        }
     }
     if (warp == kScoreWarp) tmem_alloc<CG>(smem_u32(&tmem_base_sh));  // by one full warp (of each CTA)
     __syncwarp();
@@ -673,17 +689,21 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp >= kSoftmaxWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
     if (!ok) {
-        // an unexpected base: straight to the common end
+        // an unexpected base: straight to the common end, once the first copies have landed
+        if (warp == kTmaWarp && lane == 0 && first_loads) {
+            mbar_wait_own(sbase + BAR(L::B_Q_FULL), 0);
+            mbar_wait_own(sbase + BAR(L::B_K_FULL), 0);
+        }
     } else if (warp == kTmaWarp) {
         // =============================== TMA producer
         if (lane == 0 && a.debug_no_loads == 0) {
-            // The query tile and the first keys, then keys of tile j once the score products of tile
+            // (the query tile and the first keys were requested above) Keys of tile j once the score products of tile
             // j - NSK are done, values of tile j once the value product of tile j - NSV is: the loader
             // waits on the barriers that announce those products (S_FULL, PV_DONE) instead of on
             // barriers of its own, which saves the tensor pipe two commits per tile. The score
             // products of tile t + 1 finish before the value product of tile t, so in this order no
             // wait holds up a load that could go before it.
-            int nk = 0, nv = 0;  // tiles whose keys / values were requested
+            int nk = 1, nv = 0;  // tiles whose keys / values were requested
             auto load_k = [&](int j) -> bool {
                 if (j >= n_kt) return true;
                 const int st = j % NSK;
@@ -712,12 +732,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 return true;
             };
             const uint32_t bq = sbase + BAR(L::B_Q_FULL);
-            mbar_arrive_expect_tx(bq, (SPLIT ? 2 : 1) * L::Q_ARR);
-            for (int blk = 0; blk < NB; ++blk) {  // rows outside the tensor read as zeros
-                tma_load_3d(sbase + L::OFF_Q + blk * L::Q_BLK, &maps.qh, 64 * blk, h, (int)(q0 - a.q_first), bq);
-                if (SPLIT) tma_load_3d(sbase + L::OFF_Q + L::Q_ARR + blk * L::Q_BLK, &maps.ql, 64 * blk, h, (int)(q0 - a.q_first), bq);
-            }
-            ok = load_k(0) && load_v(0) && load_k(1) && load_v(1) && load_k(2) && load_k(3) && load_k(4);
+            ok = load_v(0) && load_k(1) && load_v(1) && load_k(2) && load_k(3) && load_k(4);
             for (int t = 0; t < n_kt && ok; ++t) ok = load_k(t + 5) && load_v(t + 2);
             // let the copies requested last into each stage land before the CTA can leave
             // (earlier ones were consumed before their stage was refilled)
