@@ -89,6 +89,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <cstddef>
 #include <cstdint>
 #include <mutex>
 #include <type_traits>
@@ -152,7 +153,8 @@ struct Lay {
     static constexpr int OFF_V = NSK * K_STAGE;
     static constexpr int OFF_Q = OFF_V + NSV * V_STAGE;
     static constexpr int OFF_BARS = OFF_Q + 2 * Q_ARR;
-    static constexpr int OFF_TMEM = OFF_BARS + 248;  // after the barriers
+    static constexpr int OFF_TMEM = OFF_BARS + 232;  // after the barriers
+    static constexpr int OFF_END = OFF_TMEM + 4;     // ClosingNotes
     static constexpr int OFF_M = OFF_BARS + 256;     // float [BM]
     static constexpr int OFF_ML = OFF_M + BM * 4;    // float2 [2][BM]
     static constexpr int BYTES = OFF_ML + 2 * BM * 8;
@@ -170,9 +172,17 @@ struct Lay {
     // arrive on them, and the products' completion arrives on S_FULL and PV_DONE of both.
     static constexpr int B_Q_FULL = 0, B_K_FULL = 1, B_S_GO = B_K_FULL + NSK, B_S_FULL = B_S_GO + NSK,
                          B_V_FULL = B_S_FULL + NSK, B_P_GO = B_V_FULL + NSV, B_PV_DONE = B_P_GO + NSV,
-                         B_END = B_PV_DONE + NSV, NBAR = B_END + 2;
-    static_assert(NBAR * 8 <= 248, "barriers below the TMEM base word");
+                         NBAR = B_PV_DONE + NSV;
+    static_assert(NBAR * 8 <= 232, "barriers below the TMEM base word");
 };
+
+// What the warps of a cluster leave in each of its CTAs for the end of the kernel.
+struct ClosingNotes {
+    uint32_t bad;        // a wait gave up in either CTA
+    uint32_t scored;     // tiles whose score products were issued and committed
+    uint32_t valued;     // tiles whose value products were
+};
+static_assert(4 + sizeof(ClosingNotes) <= 256 - 232, "in the barriers' block");
 // the head-dim-128 layout (232,192 of the 232,448 bytes a CTA can have) is requested at either
 // head dim: it keeps one CTA per SM, as the CTA holds all 512 TMEM columns
 constexpr int SMEM_BYTES = Lay<128>::BYTES;
@@ -201,6 +211,11 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
     uint32_t d;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
     return d;
+}
+// *word = x in CTA `rank` of the cluster (word: the shared-memory address in this CTA)
+__device__ __forceinline__ void st_cluster(uint32_t word, uint32_t rank, uint32_t x)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(word, rank)), "r"(x) : "memory");
 }
 // All threads of the cluster's CTAs.
 __device__ __forceinline__ void cluster_sync()
@@ -613,6 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t &tmem_base_sh = *reinterpret_cast<uint32_t *>(smem + L::OFF_TMEM);
     float *const m_sh = reinterpret_cast<float *>(smem + L::OFF_M);
     float2(*const ml_sh)[BM] = reinterpret_cast<float2(*)[BM]>(smem + L::OFF_ML);
+    volatile ClosingNotes *const notes = reinterpret_cast<ClosingNotes *>(smem + L::OFF_END);
     const uint32_t sbase = smem_u32(smem);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -647,6 +663,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(smem_u32(&bars[lane]), go ? (kGroupWarps + 1) * CG : 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        if (lane == 0) {
+            notes->bad = 0u;
+            notes->scored = 0u;
+            notes->valued = 0u;
         }
         __syncwarp();
         // the query tile and the first keys at once, under the rest of the start-up (about 2,000 cycles
@@ -840,17 +861,22 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             return got;
         };
+        int issued = 0;  // tiles whose products this warp committed
         // the scores of tile j, as soon as those of tile j - 2 have been read out: they are there
         // when the group of tile j comes for them
         auto score_step = [&](auto st_c, int j) {
             if (!ok || j >= n_kt) return;
             ok = wait_all(L::B_S_GO + decltype(st_c)::value, (j / NSK) & 1);
-            if (ok) issue_s(st_c);
+            if (!ok) return;
+            issue_s(st_c);
+            issued = j + 1;
         };
         auto value_step = [&](auto st_c, int j) {
             if (!ok || j >= n_kt) return;
             ok = wait_all(L::B_P_GO + decltype(st_c)::value, (j / NSV) & 1);
-            if (ok) issue_o(st_c, j > 0 ? 1u : 0u);
+            if (!ok) return;
+            issue_o(st_c, j > 0 ? 1u : 0u);
+            issued = j + 1;
         };
         using I0 = std::integral_constant<int, 0>;
         using I1 = std::integral_constant<int, 1>;
@@ -869,11 +895,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 value_step(I1{}, j + 1);
             }
         }
-        // every product issued has to finish before TMEM is released
-        const int end = warp == kValueWarp ? L::B_END + 1 : L::B_END;
-        if (elect_one()) tc_commit<CG>(sbase + BAR(end));
-        __syncwarp();
-        mbar_wait_own(sbase + BAR(end), 0);
+        if (lane < CG) {
+            const int off = L::OFF_END + (warp == kValueWarp ? offsetof(ClosingNotes, valued) : offsetof(ClosingNotes, scored));
+            st_cluster(sbase + off, lane, (uint32_t)issued);
+        }
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
@@ -888,7 +913,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
         const float sc = a.scale_log2;
         const float v_absmax = *a.v_absmax;
-        if (lane == 0) arrive_lead(L::B_S_GO + grp);  // the group's score buffer is free for its first tile
+        if (lane == 0 && grp < n_kt) arrive_lead(L::B_S_GO + grp);  // the group's score buffer is free for its first tile
         // kept keys of word e of tile j (keys 128 (kt0 + j) + 32 e .. +31): the bitmap's word, or
         // the range suffix_lo .. i (dense: 0 .. i)
         constexpr bool kRange = DENSE || SUFFIX;
@@ -1105,13 +1130,31 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
 
-    if (!ok) atomicOr(&g_ris_tile_error, 2u);
+    if (!ok) {
+        atomicOr(&g_ris_tile_error, 2u);
+        for (int c = 0; c < CG; ++c) st_cluster(sbase + L::OFF_END + offsetof(ClosingNotes, bad), c, 1u);
+    }
     __syncwarp();
     tc_fence_before();
-    // CG = 2: neither CTA may leave while the other can still reach its shared memory or TMEM
+    // Neither CTA of a cluster may leave, or release TMEM, while a product is running or anything can
+    // still reach its shared memory. The softmax warps of each CTA have seen, in their own
+    // barriers, every commit (S_FULL of every tile, PV_DONE of every tile): nothing is under way
+    // unless a wait gave up. Then the commits still to come, as the issuing warps counted them,
+    // are waited for in each CTA before both leave.
     if constexpr (CG == 2) cluster_sync();
     __syncthreads();
     tc_fence_after();
+    if (notes->bad != 0u) {
+        if (warp == kTmaWarp && lane == 0) {
+            const int ns = (int)notes->scored, nv = (int)notes->valued;
+            for (int j = max(0, ns - NSK); j < ns; ++j) mbar_wait_own(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1);
+            for (int j = max(0, nv - NSV); j < nv; ++j) mbar_wait_own(sbase + BAR(L::B_PV_DONE + j % NSV), (j / NSV) & 1);
+        }
+        __syncwarp();
+        if constexpr (CG == 2) cluster_sync();
+        __syncthreads();
+        tc_fence_after();
+    }
     if (warp == kScoreWarp) tmem_dealloc<CG>(tmem);
 }
 
