@@ -12,8 +12,10 @@
 //   warp 8 (TMA)    loads the query tile, then streams 128-key tiles of the keys (hi parts and
 //                   corrections) and of the values (fp16) in 128-byte swizzled boxes into two
 //                   shared-memory rings, each CTA its half: a key stage is refilled as soon as its
-//                   score products are done, a value stage once its value product is;
-//   warp 11 (relay) passes what has landed in either CTA on to the barriers of the issuing warps;
+//                   score products are done, a value stage once its value product is. The copies
+//                   of both CTAs complete on barriers of the first;
+//   warp 11 (relay) (of the cluster's first CTA) passes what has landed on to the barriers of the
+//                   issuing warps;
 //   warps 9, 10     (of the cluster's first CTA) issue tcgen05.mma: warp 9 the score tile S (query
 //                   and keys from shared memory) into a double-buffered TMEM score tile, warp 10
 //                   O += P V (A = P as fp16 in TMEM, double-buffered) into the TMEM output tile,
@@ -63,6 +65,8 @@
 //                         handed over after the exponentials (it still moves at 2^8: at 2^14 the heaviest
 //                         weight of a row is less often exactly 1, and the log-sum-exp of a dense
 //                         32k layer is 5% further off);
+//                         (the waits of the softmax on what the products did are relaxed: acquiring at
+//                         cluster scope there, at 8k and 64k, made a layer 1.2-1.5% slower);
 //   1,650 / 1,870         row sums that add fp16 as it is, -infinity by predicated moves, the next
 //                         tile's scores polled for ahead of their use. Then O is rescaled after the
 //                         exponentials and the hand-over instead of before: N = 8192 230 -> 226 us.
@@ -153,7 +157,7 @@ struct Lay {
     static constexpr int OFF_V = NSK * K_STAGE;
     static constexpr int OFF_Q = OFF_V + NSV * V_STAGE;
     static constexpr int OFF_BARS = OFF_Q + 2 * Q_ARR;
-    static constexpr int OFF_TMEM = OFF_BARS + 232;  // after the barriers
+    static constexpr int OFF_TMEM = OFF_BARS + 192;  // after the barriers
     static constexpr int OFF_END = OFF_TMEM + 4;     // ClosingNotes
     static constexpr int OFF_M = OFF_BARS + 256;     // float [BM]
     static constexpr int OFF_ML = OFF_M + BM * 4;    // float2 [2][BM]
@@ -161,19 +165,26 @@ struct Lay {
     static_assert(BYTES <= 232448, "shared memory of a CTA");
     // Barriers, one of each kind per ring stage (a tile's stage is its number mod NSK or NSV), so
     // that no waiter can fall two phases behind a barrier it polls by parity:
-    //   Q_FULL          the CTA's query tile has landed (relayed with the first keys)
-    //   K_FULL, V_FULL  the CTA's part of the tile's keys / values has landed (relayed to S_GO / P_GO)
+    //   Q_FULL          the query tiles have landed (relayed with the first keys)
+    //   K_FULL, V_FULL  a tile's keys / values have landed (relayed to S_GO / P_GO)
     //   S_GO            the score products of a tile may start: its keys have landed and the scores
     //                   of the tile two before (if any) have been read out of their buffer
     //   S_FULL          they are done (and the key stage is free)
     //   P_GO            the value product may start: P is written and the values have landed
     //   PV_DONE         it is done (P's buffer and the value stage are free, O has settled)
-    // S_GO and P_GO are those of the cluster's first CTA, whose warps issue the products; both CTAs
-    // arrive on them, and the products' completion arrives on S_FULL and PV_DONE of both.
+    // S_FULL and PV_DONE of each CTA get the products' completion. The others are used in the
+    // cluster's first CTA, whose warps issue the products: the loaders of both CTAs announce
+    // their copies there and the copies complete there (each half of a tile to K_FULL or
+    // V_FULL), and the softmax warps of both arrive there.
+    //
+    // What one CTA tells the other is ordered at cluster scope: a copy's completion releases what it
+    // wrote, the relay acquires it and hands it on to the issuing warps of its own CTA; tensor
+    // memory that was read or written is ordered by the tcgen05 waits and fences around the arrival and
+    // the wait, which themselves need no more than the scope (see mbar_arrive_cluster).
     static constexpr int B_Q_FULL = 0, B_K_FULL = 1, B_S_GO = B_K_FULL + NSK, B_S_FULL = B_S_GO + NSK,
                          B_V_FULL = B_S_FULL + NSK, B_P_GO = B_V_FULL + NSV, B_PV_DONE = B_P_GO + NSV,
                          NBAR = B_PV_DONE + NSV;
-    static_assert(NBAR * 8 <= 232, "barriers below the TMEM base word");
+    static_assert(NBAR * 8 <= 192, "barriers below the TMEM base word");
 };
 
 // What the warps of a cluster leave in each of its CTAs for the end of the kernel.
@@ -181,8 +192,9 @@ struct ClosingNotes {
     uint32_t bad;        // a wait gave up in either CTA
     uint32_t scored;     // tiles whose score products were issued and committed
     uint32_t valued;     // tiles whose value products were
+    uint32_t keys[2], values[2];  // tiles whose keys / values each CTA requested (in the first CTA)
 };
-static_assert(4 + sizeof(ClosingNotes) <= 256 - 232, "in the barriers' block");
+static_assert(4 + sizeof(ClosingNotes) <= 256 - 192, "in the barriers' block");
 // the head-dim-128 layout (232,192 of the 232,448 bytes a CTA can have) is requested at either
 // head dim: it keeps one CTA per SM, as the CTA holds all 512 TMEM columns
 constexpr int SMEM_BYTES = Lay<128>::BYTES;
@@ -198,13 +210,13 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // Arrival on a barrier of any CTA of the cluster (shared::cluster address, see cluster_addr). What
-// it announces is tensor memory that was read or written (ordered by tcgen05.wait and
-// tcgen05.fence) or a copy that landed, not this thread's memory accesses: releasing those at
-// cluster scope took 1,000 cycles and more per arrival (a tile of a 32k dense layer took
-// 3,130 cycles instead of 1,720).
+// it announces is tensor memory that was read or written, which tcgen05.wait and the tcgen05 fences on
+// both sides order, and nothing that this thread read or wrote itself: relaxed. (Releasing its
+// accesses at cluster scope took 1,000 cycles and more per arrival: 3,130 cycles a tile of a 32k dense
+// layer instead of 1,720.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
 {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
 {
@@ -218,64 +230,124 @@ __device__ __forceinline__ void st_cluster(uint32_t word, uint32_t rank, uint32_
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(word, rank)), "r"(x) : "memory");
 }
 // All threads of the cluster's CTAs.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
+// Announce `bytes` to come on the barrier; CG = 2: a barrier of either CTA (shared::cluster address),
+// relaxed, as nothing of this thread's is handed over.
+template <int CG>
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
 {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    if constexpr (CG == 1)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    else
+        asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
+                     : "memory");
 }
+// Waits acquire at the scope of those who arrive: the cluster's two CTAs and their copies (CG = 2). TMEM:
+// what is waited for is tensor memory that products read or wrote, which the tcgen05 fence after the
+// wait orders; relaxed, at the same scope.
+template <int CG, bool TMEM = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
+    if constexpr (CG == 2 && TMEM)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    else if constexpr (CG == 1)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
     return ok != 0;
 }
-// Bounded wait for this CTA's own asynchronous work (copies or products already issued):
-// about 2^31 cycles at most, whatever other CTAs reported.
+// Bounded wait for asynchronous work already issued (copies or products): about 2^31 cycles at most,
+// whatever other CTAs reported.
+template <int CG>
 __device__ __forceinline__ bool mbar_wait_own(uint32_t bar, uint32_t parity)
 {
     const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
+    while (!mbar_try_wait<CG>(bar, parity))
         if (clock64() - t0 > (1LL << 31)) return false;
     return true;
 }
 
 // Whether the phase has completed by now: asked ahead of the wait, so that a completed one costs
 // no round trip to the barrier at the point of use
+template <int CG, bool TMEM = false>
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
+    if constexpr (CG == 2 && TMEM)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    else if constexpr (CG == 1)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
     return ok != 0;
 }
 
 // Bounded wait (`limit` cycles, about 2^31 unless a test lowers it); false if the phase did
 // not complete in time or another CTA already gave up.
+template <int CG, bool TMEM = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long limit)
 {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<CG, TMEM>(bar, parity)) return true;
     const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
+    while (!mbar_try_wait<CG, TMEM>(bar, parity)) {
         if (clock64() - t0 > limit) return false;
         if (*reinterpret_cast<volatile unsigned int *>(&g_ris_tile_error) != 0u) return false;
     }
     return true;
 }
 
+// Copy a box into this CTA's shared memory. CG = 2: complete on a barrier of either CTA of the pair.
+template <int CG>
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, uint32_t bar)
 {
+    if constexpr (CG == 2)
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 "
+        "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+        : "memory");
+    else
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cta.global.tile.mbarrier::complete_tx::bytes "
         "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
@@ -658,37 +730,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == kTmaWarp) {
         static_assert(L::NBAR <= 32, "a lane per barrier");
         if (lane < L::NBAR) {
-            // S_GO, P_GO: the group's warps and the relay, of each CTA
+            // S_GO, P_GO: the group's warps of each CTA and the relay; S_FULL, PV_DONE: the commit; the
+            // copies' barriers: the loader of each CTA
             const bool go = (lane >= L::B_S_GO && lane < L::B_S_GO + NSK) || (lane >= L::B_P_GO && lane < L::B_P_GO + NSV);
-            mbar_init(smem_u32(&bars[lane]), go ? (kGroupWarps + 1) * CG : 1);
+            const bool done = (lane >= L::B_S_FULL && lane < L::B_S_FULL + NSK) || lane >= L::B_PV_DONE;
+            mbar_init(smem_u32(&bars[lane]), go ? kGroupWarps * CG + 1 : done ? 1 : CG);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
-        if (lane == 0) {
-            notes->bad = 0u;
-            notes->scored = 0u;
-            notes->valued = 0u;
-        }
+        if (lane < (int)(sizeof(ClosingNotes) / 4)) reinterpret_cast<volatile uint32_t *>(smem + L::OFF_END)[lane] = 0u;
         __syncwarp();
-        // the query tile and the first keys at once, under the rest of the start-up (about 2,000 cycles
-        // of TMEM allocation and cluster barrier): only this CTA's own barriers are involved
-        if (lane == 0 && first_loads) {
-            const uint32_t bq = sbase + L::OFF_BARS + 8 * L::B_Q_FULL, bk = sbase + L::OFF_BARS + 8 * L::B_K_FULL;
-            const int key = kt0 * BN + L::KROWS * rank;
-            mbar_arrive_expect_tx(bq, (SPLIT ? 2 : 1) * L::Q_ARR);
-            mbar_arrive_expect_tx(bk, (SPLIT ? 2 : 1) * L::K_ARR);
-            for (int blk = 0; blk < NB; ++blk) {
-                tma_load_3d(sbase + L::OFF_Q + blk * L::Q_BLK, &maps.qh, 64 * blk, h, (int)(q0 - a.q_first), bq);
-                if (SPLIT) tma_load_3d(sbase + L::OFF_Q + L::Q_ARR + blk * L::Q_BLK, &maps.ql, 64 * blk, h, (int)(q0 - a.q_first), bq);
-                tma_load_3d(sbase + L::OFF_K + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
-                if (SPLIT) tma_load_3d(sbase + L::OFF_K + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
-            }
+    }
+    // The barriers of both CTAs are initialised once this cluster barrier is passed. (That the other CTA's
+    // tensor memory is allocated before a product writes to it follows from its softmax warps'
+    // first arrivals.)
+    if constexpr (CG == 2) cluster_arrive();
+    if (warp == kScoreWarp) tmem_alloc<CG>(smem_u32(&tmem_base_sh));  // by one full warp (of each CTA)
+    if constexpr (CG == 2) cluster_wait();
+    const uint32_t lead = CG == 2 ? cluster_addr(sbase, 0) : sbase;  // the issuing CTA's shared memory
+    constexpr auto BAR = [](int i) { return (uint32_t)(L::OFF_BARS + 8 * i); };
+    // the query tile and the first keys at once, under the rest of the start-up (about 2,000 cycles, the
+    // TMEM allocation most of them)
+    if (warp == kTmaWarp && lane == 0 && first_loads) {
+        const uint32_t bq = lead + BAR(L::B_Q_FULL), bk = lead + BAR(L::B_K_FULL);
+        const int key = kt0 * BN + L::KROWS * rank;
+        mbar_arrive_expect_tx<CG>(bq, (SPLIT ? 2 : 1) * L::Q_ARR);
+        mbar_arrive_expect_tx<CG>(bk, (SPLIT ? 2 : 1) * L::K_ARR);
+        for (int blk = 0; blk < NB; ++blk) {
+            const int row = (int)(q0 - a.q_first);
+            tma_load_3d<CG>(sbase + L::OFF_Q + blk * L::Q_BLK, &maps.qh, 64 * blk, h, row, bq);
+            if (SPLIT) tma_load_3d<CG>(sbase + L::OFF_Q + L::Q_ARR + blk * L::Q_BLK, &maps.ql, 64 * blk, h, row, bq);
+            tma_load_3d<CG>(sbase + L::OFF_K + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
+            if (SPLIT) tma_load_3d<CG>(sbase + L::OFF_K + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
         }
     }
-    if (warp == kScoreWarp) tmem_alloc<CG>(smem_u32(&tmem_base_sh));  // by one full warp (of each CTA)
     __syncwarp();
     tc_fence_before();
-    if constexpr (CG == 2) cluster_sync();
     __syncthreads();
     tc_fence_after();
     // all 512 columns: the allocation starts at TMEM address 0, so every address below is a
@@ -696,8 +773,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t T_S0 = 0, T_O = T_S0 + 2 * BN, T_P0 = T_O + DT;
     static_assert(T_P0 + BN <= kTmemCols, "TMEM columns");
     const uint32_t tmem = tmem_base_sh;
-    constexpr auto BAR = [](int i) { return (uint32_t)(L::OFF_BARS + 8 * i); };
-    const uint32_t lead = CG == 2 ? cluster_addr(sbase, 0) : sbase;  // the issuing CTA's shared memory
     auto arrive_lead = [&](int bar) {
         if constexpr (CG == 2)
             mbar_arrive_cluster(lead + BAR(bar));
@@ -709,17 +784,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (warp >= kSoftmaxWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
-    if (!ok) {
-        // an unexpected base: straight to the common end, once the first copies have landed
-        if (warp == kTmaWarp && lane == 0 && first_loads) {
-            mbar_wait_own(sbase + BAR(L::B_Q_FULL), 0);
-            mbar_wait_own(sbase + BAR(L::B_K_FULL), 0);
-        }
-    } else if (warp == kTmaWarp) {
+    if (warp == kTmaWarp) {
         // =============================== TMA producer
-        if (lane == 0 && a.debug_no_loads == 0) {
-            // (the query tile and the first keys were requested above) Keys of tile j once the score products of tile
-            // j - NSK are done, values of tile j once the value product of tile j - NSV is: the loader
+        if (lane == 0 && first_loads) {
+            // (The query tile and the first keys were requested above.) Keys of tile j once the score
+            // products of tile j - NSK are done, values of tile j once the value product of tile j - NSV is: the loader
             // waits on the barriers that announce those products (S_FULL, PV_DONE) instead of on
             // barriers of its own, which saves the tensor pipe two commits per tile. The score
             // products of tile t + 1 finish before the value product of tile t, so in this order no
@@ -728,14 +797,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             auto load_k = [&](int j) -> bool {
                 if (j >= n_kt) return true;
                 const int st = j % NSK;
-                if (j >= NSK && !mbar_wait(sbase + BAR(L::B_S_FULL + st), (j / NSK - 1) & 1, wl)) return false;
-                const uint32_t bk = sbase + BAR(L::B_K_FULL + st);
+                if (j >= NSK && !mbar_wait<CG>(sbase + BAR(L::B_S_FULL + st), (j / NSK - 1) & 1, wl)) return false;
+                const uint32_t bk = lead + BAR(L::B_K_FULL + st);
                 const uint32_t dk = sbase + L::OFF_K + st * L::K_STAGE;
                 const int key = (kt0 + j) * BN + L::KROWS * rank;
-                mbar_arrive_expect_tx(bk, (SPLIT ? 2 : 1) * L::K_ARR);
+                mbar_arrive_expect_tx<CG>(bk, (SPLIT ? 2 : 1) * L::K_ARR);
                 for (int blk = 0; blk < NB; ++blk) {
-                    tma_load_3d(dk + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
-                    if (SPLIT) tma_load_3d(dk + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
+                    tma_load_3d<CG>(dk + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
+                    if (SPLIT) tma_load_3d<CG>(dk + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
                 }
                 nk = j + 1;
                 return true;
@@ -743,48 +812,45 @@ __global__ void __launch_bounds__(kThreads, 1)
             auto load_v = [&](int j) -> bool {
                 if (j >= n_kt) return true;
                 const int st = j % NSV;
-                if (j >= NSV && !mbar_wait(sbase + BAR(L::B_PV_DONE + st), (j / NSV - 1) & 1, wl)) return false;
-                const uint32_t bv = sbase + BAR(L::B_V_FULL + st);
+                if (j >= NSV && !mbar_wait<CG>(sbase + BAR(L::B_PV_DONE + st), (j / NSV - 1) & 1, wl)) return false;
+                const uint32_t bv = lead + BAR(L::B_V_FULL + st);
                 const uint32_t dv = sbase + L::OFF_V + st * L::V_STAGE;
-                mbar_arrive_expect_tx(bv, L::V_STAGE);
+                mbar_arrive_expect_tx<CG>(bv, L::V_STAGE);
                 for (int blk = 0; blk < NB / CG; ++blk)
-                    tma_load_3d(dv + blk * L::V_BLK, &maps.v, 64 * (blk + rank), g, (kt0 + j) * BN, bv);
+                    tma_load_3d<CG>(dv + blk * L::V_BLK, &maps.v, 64 * (blk + rank), g, (kt0 + j) * BN, bv);
                 nv = j + 1;
                 return true;
             };
-            const uint32_t bq = sbase + BAR(L::B_Q_FULL);
-            ok = load_v(0) && load_k(1) && load_v(1) && load_k(2) && load_k(3) && load_k(4);
+            ok = ok && load_v(0) && load_k(1) && load_v(1) && load_k(2) && load_k(3) && load_k(4);
             for (int t = 0; t < n_kt && ok; ++t) ok = load_k(t + 5) && load_v(t + 2);
-            // let the copies requested last into each stage land before the CTA can leave
-            // (earlier ones were consumed before their stage was refilled)
-            mbar_wait_own(bq, 0);
-            for (int j = nk - NSK; j < nk; ++j)
-                if (j >= 0) mbar_wait_own(sbase + BAR(L::B_K_FULL + j % NSK), (j / NSK) & 1);
-            for (int j = nv - NSV; j < nv; ++j)
-                if (j >= 0) mbar_wait_own(sbase + BAR(L::B_V_FULL + j % NSV), (j / NSV) & 1);
+            // (that the copies requested last have landed before a CTA leaves: see the end)
+            st_cluster(sbase + L::OFF_END + offsetof(ClosingNotes, keys) + 4 * rank, 0, (uint32_t)nk);
+            st_cluster(sbase + L::OFF_END + offsetof(ClosingNotes, values) + 4 * rank, 0, (uint32_t)nv);
             static_assert(NSK == 4 && NSV == 2, "the order of the loads and of the relay");
         }
+    } else if (!ok || rank != 0) {
+        // an unexpected base: straight to the common end; and the second CTA has nothing to issue
     } else if (warp == kRelayWarp) {
         // =============================== relay: what has landed, to the barriers that the issuing
         // warps wait on, in the order of the loads; so each of them waits on one barrier per tile
         if (lane == 0) {
             auto relay_k = [&](int j) -> bool {
                 if (j >= n_kt) return true;
-                if (!mbar_wait(sbase + BAR(L::B_K_FULL + j % NSK), (j / NSK) & 1, wl)) return false;
-                arrive_lead(L::B_S_GO + j % NSK);
+                if (!mbar_wait<CG>(sbase + BAR(L::B_K_FULL + j % NSK), (j / NSK) & 1, wl)) return false;
+                mbar_arrive(sbase + BAR(L::B_S_GO + j % NSK));
                 return true;
             };
             auto relay_v = [&](int j) -> bool {
                 if (j >= n_kt) return true;
-                if (!mbar_wait(sbase + BAR(L::B_V_FULL + j % NSV), (j / NSV) & 1, wl)) return false;
-                arrive_lead(L::B_P_GO + j % NSV);
+                if (!mbar_wait<CG>(sbase + BAR(L::B_V_FULL + j % NSV), (j / NSV) & 1, wl)) return false;
+                mbar_arrive(sbase + BAR(L::B_P_GO + j % NSV));
                 return true;
             };
-            ok = mbar_wait(sbase + BAR(L::B_Q_FULL), 0, wl) && relay_k(0) && relay_v(0) && relay_k(1) && relay_v(1) &&
+            ok = mbar_wait<CG>(sbase + BAR(L::B_Q_FULL), 0, wl) && relay_k(0) && relay_v(0) && relay_k(1) && relay_v(1) &&
                  relay_k(2) && relay_k(3) && relay_k(4);
             for (int t = 0; t < n_kt && ok; ++t) ok = relay_k(t + 5) && relay_v(t + 2);
         }
-    } else if (rank == 0) {
+    } else {
         // =============================== product issuers (of the cluster's first CTA, for both): one
         // warp for the scores, one for the value products, so that neither's waits (about 100
         // cycles each even on a completed phase) leave the tensor pipe without queued work.
@@ -857,7 +923,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
         };
         auto wait_all = [&](int bar, int parity) -> bool {
-            const bool got = __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(bar), parity, wl));
+            const bool got = __all_sync(0xFFFFFFFFu, mbar_wait<CG>(sbase + BAR(bar), parity, wl));
             tc_fence_after();
             return got;
         };
@@ -955,7 +1021,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool s_full = false;  // seen at the end of the last tile: a poll takes 200 cycles even if it succeeds
         for (int j = grp; j < n_kt; j += 2) {
             if (!kRange) mask_words(j + 4, nnw);
-            if (ok) ok = __all_sync(0xFFFFFFFFu, s_full || mbar_wait(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1, wl));
+            if (ok) ok = __all_sync(0xFFFFFFFFu, s_full || mbar_wait<CG, true>(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1, wl));
             tc_fence_after();
             uint32_t su[2][64];
             tmem_issue64(T_S0 + grp * BN + lane_off, su[0]);
@@ -970,6 +1036,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             pin64(su[1]);
             tc_fence_before();
             __syncwarp();
+            tc_fence_before();
             if (lane == 0 && j + 2 < n_kt) arrive_lead(L::B_S_GO + (j + 2) % NSK);
             float sv[BN];
 #pragma unroll
@@ -1009,7 +1076,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const float m_ref = upd ? mx : m_prev;
             // the value product of tile t is done (t < 0: nothing to wait for)
             auto pv_done = [&](int t) -> bool {
-                return t < 0 || __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
+                return t < 0 || __all_sync(0xFFFFFFFFu, mbar_wait<CG, true>(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
             };
             const bool scale_o = upd && m_prev != -INFINITY;
             const bool any_scale = __any_sync(0xFFFFFFFFu, scale_o);
@@ -1071,18 +1138,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t tp = T_P0 + grp * (BN / 2) + lane_off;
             tmem_st32(tp, hw);
             tmem_st32(tp + 32, hw + 32);
-            s_full = j + 2 < n_kt && mbar_test(sbase + BAR(L::B_S_FULL + (j + 2) % NSK), ((j + 2) / NSK) & 1);
+            s_full = j + 2 < n_kt && mbar_test<CG, true>(sbase + BAR(L::B_S_FULL + (j + 2) % NSK), ((j + 2) / NSK) & 1);
             l += (lsum[0] + lsum[2]) + (lsum[1] + lsum[3]);
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
+            tc_fence_before();
             if (lane == 0) arrive_lead(L::B_P_GO + grp);
         }
         // the row's maximum and sum from both threads
         ml_sh[grp][r] = make_float2(m_own, l);
         ok = !pair_or(9 + wq, !ok);
         for (int t = max(0, n_kt - 2); t < n_kt && ok; ++t)  // in order, as above
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait<CG>(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
         if (ok) {
             tc_fence_after();
             const float2 ma = ml_sh[0][r], mb = ml_sh[1][r];
@@ -1138,17 +1206,33 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     // Neither CTA of a cluster may leave, or release TMEM, while a product is running or anything can
     // still reach its shared memory. The softmax warps of each CTA have seen, in their own
-    // barriers, every commit (S_FULL of every tile, PV_DONE of every tile): nothing is under way
-    // unless a wait gave up. Then the commits still to come, as the issuing warps counted them,
-    // are waited for in each CTA before both leave.
+    // barriers, every commit (S_FULL of every tile, PV_DONE of every tile), and so the end of every copy:
+    // nothing is under way unless a wait gave up. Then the copies and commits still to come, as the
+    // loaders and the issuing warps counted them, are waited for before both CTAs leave. (What one
+    // loader requested and the other did not is announced here in its place. A tile is requested only
+    // after the products on its stage's last tile, so no count is behind by more than the ring, and no
+    // barrier by more than one phase.)
     if constexpr (CG == 2) cluster_sync();
     __syncthreads();
     tc_fence_after();
     if (notes->bad != 0u) {
         if (warp == kTmaWarp && lane == 0) {
+            auto landed = [&](int bar, int stages, int n0, int n1) {
+                const int n = max(n0, n1);
+                for (int j = max(0, n - stages); j < n; ++j) {
+                    if (j >= min(n0, n1)) mbar_arrive(sbase + BAR(bar + j % stages));
+                    mbar_wait_own<CG>(sbase + BAR(bar + j % stages), (j / stages) & 1);
+                }
+            };
+            if (rank == 0) {
+                constexpr int R1 = CG - 1;
+                if (notes->keys[0] > 0u) mbar_wait_own<CG>(sbase + BAR(L::B_Q_FULL), 0);
+                landed(L::B_K_FULL, NSK, (int)notes->keys[0], (int)notes->keys[R1]);
+                landed(L::B_V_FULL, NSV, (int)notes->values[0], (int)notes->values[R1]);
+            }
             const int ns = (int)notes->scored, nv = (int)notes->valued;
-            for (int j = max(0, ns - NSK); j < ns; ++j) mbar_wait_own(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1);
-            for (int j = max(0, nv - NSV); j < nv; ++j) mbar_wait_own(sbase + BAR(L::B_PV_DONE + j % NSV), (j / NSV) & 1);
+            for (int j = max(0, ns - NSK); j < ns; ++j) mbar_wait_own<CG>(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1);
+            for (int j = max(0, nv - NSV); j < nv; ++j) mbar_wait_own<CG>(sbase + BAR(L::B_PV_DONE + j % NSV), (j / NSV) & 1);
         }
         __syncwarp();
         if constexpr (CG == 2) cluster_sync();

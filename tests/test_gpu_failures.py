@@ -138,6 +138,41 @@ def test_tile_wait_gives_up_and_context_survives():
     m.free()
 
 
+@pytest.mark.parametrize("N,Hq,Hkv,D,mode,d", [(2000, 4, 2, 128, 0, 0.5), (1300, 6, 2, 128, 2, 1.0), (1300, 4, 2, 64, 0, 0.5)],
+                         ids=["head_pairs", "tile_pairs", "one_cta"])
+def test_tile_gives_up_with_copies_and_products_under_way(N, Hq, Hkv, D, mode, d):
+    """Waits that end early at any point of the pipeline, with the loader running: the copies and products
+    under way are waited for, and the same call afterwards gives what it gave before."""
+    (q, k, v), _ = make_inputs(N, Hq, Hkv, D, seed=29, outliers=True)
+    rope = ris.rope_cfg(3, 1e6, 256)
+    with ris.ris_mask_generate(N, Hkv, mode, d, [1]) as m:
+        assert ris.ris_attention_design(m, torch.bfloat16, D) == 2  # the tile kernel
+
+        def call():
+            return ris.ris_attention_masked(m, q, k, v, rope=rope, out_dtype=torch.float32)
+        ref = call()
+        torch.cuda.synchronize()
+        ris.ris_device_status()
+        gave_up = 0
+        for limit in (1, 30, 100, 300, 600, 1000, 2000, 4000):
+            try:
+                ris.ris_debug_tile_stall(False, limit)
+                call()
+                torch.cuda.synchronize()
+            finally:
+                ris.ris_debug_tile_stall(False, 0)
+            try:
+                ris.ris_device_status()
+            except ris.RisError as e:
+                assert e.status == ris.RIS_ERR_DEVICE_TIMEOUT
+                gave_up += 1
+            again = call()
+            torch.cuda.synchronize()
+            ris.ris_device_status()
+            assert torch.equal(again, ref), f"limit {limit}"
+        assert gave_up > 0
+
+
 def test_shutdown_releases_caches_and_library_stays_usable():
     N, Hq, Hkv, D = 900, 6, 2, 128
     (q, k, v), _ = make_inputs(N, Hq, Hkv, D, seed=5, outliers=True)
