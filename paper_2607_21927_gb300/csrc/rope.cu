@@ -409,7 +409,10 @@ cudaError_t launch_fp8_prep(const Fp8PrepArgs &a, cudaStream_t s)
     if (a.D != kPrepDim) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(a.bounds, 0, 3 * sizeof(float), s);
     if (e != cudaSuccess) return e;
-    const int64_t pieces = a.q_rows * a.Hq * (a.D / 16);  // of the largest tensor
+    // pieces of the largest tensor: q of a whole layer as a rule, but k and v where q holds a few local rows, and v
+    // where every query head has its own KV head
+    const int64_t pieces = std::max(std::max(a.q_rows * a.Hq, a.N * a.Hkv) * (a.D / 16),
+                                    a.v16 != nullptr ? a.N * a.Hkv * (a.D / 8) : 0);
     const int64_t need = (pieces + kBoundThreads - 1) / kBoundThreads;
     k_fp8_bounds<<<(unsigned)std::min<int64_t>(std::max<int64_t>(need, 1), kBoundBlocks), kBoundThreads, 0, s>>>(a);
     // at least six CTAs per SM, as far as there are heads to slice
