@@ -5,10 +5,10 @@
 // causal bitmap row with all seeds OR-merged in registers (the paper's streaming merge,
 // without ever holding a seed's mask), then compacted into ascending per-row key lists.
 //
-//   k_mask_bits : per (mask, row) CTA, per group of 4 keys: one Philox4x32-10 call per seed, the
-//                 smallest word over the seeds against the threshold, then per 32-key word the
-//                 forced window/anchors, Structural block clique and causal cut; writes the
-//                 word and the row's key count.
+//   k_mask_bits : per (mask, row) CTA, per group of 4 keys: one Philox4x32-10 call per seed until every key
+//                 of the warp's step is kept, the smallest word over the seeds against the
+//                 threshold, then per 32-key word the forced window/anchors, Structural block
+//                 clique and causal cut; writes the word and the row's key count.
 //   k_mask_draws: index-draw sampler only: per (mask, row) CTA, the row's index draws of
 //                 every seed (one Philox call = 4 draws), j = floor(u N / 2^32), kept when
 //                 j < i by an atomic OR into the zeroed bitmap row; k_mask_bits then ORs the
@@ -18,6 +18,7 @@
 //
 // Integer-only; every decision is an exact comparison of a 32-bit word with a host-resolved
 // 64-bit threshold, so the result is bit-exact across devices and hosts.
+#include <cmath>
 #include <cstdint>
 
 #include "ris_internal.h"
@@ -61,16 +62,19 @@ struct RowDraws {
 };
 
 // Smallest word over the seeds s0 .. s1-1 of each of the 4 keys of the groups g .. g + U - 1 (keys
-// 4 g .. 4 g + 4 U - 1): a key is kept by some seed iff this minimum is below the threshold.
+// 4 g .. 4 g + 4 U - 1): a key is kept by some seed iff this minimum is at most tm1. `forced`: the draws of these
+// keys do not matter, and whatever is returned for them is kept. A warp whose keys are all kept leaves the loop
+// over seeds: it asks after `first_vote` seeds and then every kVoteSeeds.
 //
 // Philox4x32-10 as in philox4x32_10 above, with what the 10 rounds of a row's calls have in common
 // taken out of the loop over seeds (SEEDS a pass; 0: one seed in all, s0, without a loop or minima). Round 1 multiplies the group (word 0) and the stream (word 2),
 // neither of which depends on the seed; its results z, w depend on the group only (key word 1 is
 // the head key) and x, y on the row and seed only. So the second product of round 2 depends on the
 // group only and the first on the seed only: per call 8 rounds of two products remain, 16 of 20.
+constexpr int kVoteSeeds = 4;
 template <int U, int SEEDS>
 __device__ __forceinline__ void min_words(const MaskBitsArgs &a, const RowDraws &d, uint32_t g, int s0, int s1,
-                                          uint32_t (&best)[U][4])
+                                          uint32_t tm1, bool forced, int first_vote, uint32_t (&best)[U][4])
 {
     uint32_t hx[U], y2[U], wz[U];  // x2 but for key word 0, y2, z2 but for the seed's product
 #pragma unroll
@@ -81,11 +85,9 @@ __device__ __forceinline__ void min_words(const MaskBitsArgs &a, const RowDraws 
         y2[u] = (uint32_t)p1;
         wz[u] = (uint32_t)p0 ^ (d.k1 + 0xBB67AE85u);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) best[u][e] = 0xFFFFFFFFu;
+        for (int e = 0; e < 4; ++e) best[u][e] = SEEDS > 0 && forced ? 0u : 0xFFFFFFFFu;
     }
-    const int end = SEEDS == 0 ? s0 + 1 : s1;
-#pragma unroll(SEEDS == 0 ? 1 : SEEDS)
-    for (int s = s0; s < end; ++s) {
+    auto seed_pass = [&](int s) {
         uint32_t k0 = a.seeds.v[s], k1 = d.k1 + 0xBB67AE85u;
         const uint64_t ps = (uint64_t)0xD2511F53u * (d.s_hi ^ d.i ^ k0);
         k0 += 0x9E3779B9u;
@@ -111,6 +113,23 @@ __device__ __forceinline__ void min_words(const MaskBitsArgs &a, const RowDraws 
             best[u][1] = min(best[u][1], c[u].y);
             best[u][2] = min(best[u][2], c[u].z);
             best[u][3] = min(best[u][3], c[u].w);
+        }
+    };
+    if constexpr (SEEDS == 0) {
+        seed_pass(s0);
+    } else {
+        int s = s0, stop = min(s1, s0 + first_vote);
+        for (;;) {
+#pragma unroll SEEDS
+            for (; s < stop; ++s) seed_pass(s);
+            if (s >= s1) break;
+            uint32_t worst = 0u;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) worst = max(worst, best[u][e]);
+            if (__all_sync(0xFFFFFFFFu, worst <= tm1)) break;
+            stop = min(s1, s + kVoteSeeds);
         }
     }
 }
@@ -152,12 +171,14 @@ __device__ __forceinline__ RowTask row_task(const MaskBitsArgs &a, uint32_t m, i
 // One warp, 16 words (512 keys) from word w0 on: lane l takes the 16 keys of half a word, groups
 // 4 l .. 4 l + 3 of the step's 128, and its neighbour the other half. Returns the lane's kept keys.
 template <int SEEDS>
-__device__ __forceinline__ int row_step(const MaskBitsArgs &a, const RowTask &t, int w0, int lane)
+__device__ __forceinline__ int row_step(const MaskBitsArgs &a, const RowTask &t, int w0, int lane, int first_vote)
 {
     uint32_t word = 0u;
-    if (8 * w0 < t.ng) {
+    if (8 * w0 < t.ng && 32u * (uint32_t)(w0 + 16) > (uint32_t)a.A) {  // some key of the step is not forced
         uint32_t best[4][4];
-        min_words<4, SEEDS>(a, t.d, (uint32_t)(8 * w0 + 4 * lane), t.s0, t.s1, best);
+        const int g = 8 * w0 + 4 * lane;
+        const bool forced = g >= t.ng || 4u * (uint32_t)(g + 4) <= (uint32_t)a.A;
+        min_words<4, SEEDS>(a, t.d, (uint32_t)g, t.s0, t.s1, t.tm1, forced, first_vote, best);
 #pragma unroll
         for (int e = 0; e < 16; ++e) word |= best[e >> 2][e & 3] <= t.tm1 ? 1u << e : 0u;
     }
@@ -182,7 +203,7 @@ __device__ __forceinline__ int row_step(const MaskBitsArgs &a, const RowTask &t,
 // per word, 21.1 with rounds 1 and 2 taken out, 19.6 now (1.5 calls per clock and SM). SEEDS = 0, one seed: eight
 // CTAs per SM, a row's other work counts.
 template <int SEEDS>
-__global__ void __launch_bounds__(kBitsThreads, SEEDS > 0 ? 1 : 8) k_mask_bits(const MaskBitsArgs a)
+__global__ void __launch_bounds__(kBitsThreads, SEEDS > 0 ? 1 : 8) k_mask_bits(const MaskBitsArgs a, int first_vote)
 {
     const uint32_t m = blockIdx.x % (uint32_t)a.n_masks;
     const bool one = a.single_row >= 0;
@@ -190,7 +211,7 @@ __global__ void __launch_bounds__(kBitsThreads, SEEDS > 0 ? 1 : 8) k_mask_bits(c
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const RowTask t = row_task(a, m, i);
     int count = 0;
-    for (int w0 = 16 * warp; w0 < t.nw; w0 += 16 * (kBitsThreads / 32)) count += row_step<SEEDS>(a, t, w0, lane);
+    for (int w0 = 16 * warp; w0 < t.nw; w0 += 16 * (kBitsThreads / 32)) count += row_step<SEEDS>(a, t, w0, lane, first_vote);
     // block reduction of the row count
     __shared__ int red[kBitsThreads / 32];
     count = __reduce_add_sync(0xFFFFFFFFu, count);
@@ -225,7 +246,7 @@ __global__ void __launch_bounds__(kBitsThreads, 6) k_mask_bits_one(const MaskBit
         if (at < steps) {
             const RowTask t = row_task(a, m, i);
             int count = 0;
-            for (; at < steps; at += kBitsThreads / 32) count += row_step<0>(a, t, 16 * at, lane);
+            for (; at < steps; at += kBitsThreads / 32) count += row_step<0>(a, t, 16 * at, lane, 0);
             count = __reduce_add_sync(0xFFFFFFFFu, count);
             if (lane == 0) atomicAdd(&total[q], count);
         }
@@ -425,12 +446,20 @@ cudaError_t launch_mask_bits(const MaskBitsArgs &a, cudaStream_t s)
     const int seeds = a.per_seed ? 1 : a.n_seeds;
     // four rows per CTA only if that leaves sixteen CTAs per SM: below, rows in flight count for more
     // (N = 2048, one seed: 7.3 us against 6.4)
+    // Seeds after which one warp step of 512 keys in e^3 is full: 512 (1 - hit)^s = 3, hit the chance that a
+    // seed keeps a key. Asking costs about a tenth of a seed's pass, so sparse masks (1%: 512 seeds) never ask,
+    // and dense ones first where it may help. Mask of N = 8192, every seed drawn / asking: 50% x 256 seeds
+    // 4.86 / 0.54 ms, 10% x 256 4.86 / 1.52, 30% x 70 1.53 / 0.67, 10% x 70 1.54 / 1.42; 1% x 70 with every key an
+    // anchor 1.53 / 0.29. (A skip per group of four keys and thread: 1.24, 2.31, 0.85, 1.73; 0.46.)
+    const double hit = (double)a.thr / 4294967296.0;
+    const double full = hit >= 1.0 ? 1.0 : std::ceil(std::log(512.0 / 3.0) / -std::log1p(-hit));
+    const int first_vote = a.thr == 0 || full > kMaxSeeds ? kMaxSeeds : (int)full;
     if (seeds == 1 && a.single_row < 0 && blocks >= (int64_t)kOneSeedRows * 16 * 152)
         k_mask_bits_one<<<(unsigned)((blocks + kOneSeedRows - 1) / kOneSeedRows), kBitsThreads, 0, s>>>(a);
     else if (seeds == 1)
-        k_mask_bits<0><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
+        k_mask_bits<0><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a, first_vote);
     else
-        k_mask_bits<2><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a);
+        k_mask_bits<2><<<(unsigned)blocks, kBitsThreads, 0, s>>>(a, first_vote);
     note_launch();
     return cudaGetLastError();
 }
