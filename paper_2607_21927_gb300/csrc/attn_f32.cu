@@ -14,14 +14,14 @@
 // Products and sums run as packed pairs of fp32 (fma.rn.f32x2, rounded as the scalar operation):
 // half the issue slots. Bound by the L2 rows (2 D 4 B per pair and KV head) and the FFMA pipe
 // alike; residency hides the load latency: three CTAs of four warps per SM, four with one or two
-// heads in a group (layer call of one head at N = 2048: 31.4 against 33.3 us; six heads at N = 6007:
-// 291 us with three, 314 with two, 401 with four, which spill).
-// Layer calls, before (one lane per key row, 32 lines per load, groups padded to eight heads) -> now:
-// 12 / 2 heads of 128, N = 6007, 4.9% of the pairs: 492 -> 274 us; one head, N = 2048, 5%: 50 -> 28 us (17 and 3 us of them by the
-// launch that rotates q and k together and the shorter host path).
+// heads in a group. (With six heads at N = 6007 two CTAs were 8% slower, four, which spill, 38%; one head at
+// N = 2048 is 6% faster with four.) A lane per key row instead, 32 lines per load and groups padded to
+// eight heads, took 492 us for 12 / 2 heads of 128, N = 6007, 4.9% of the pairs, and 50 us for one head,
+// N = 2048, 5%; these layer calls take 249 and 28-31 us.
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "attn_common.cuh"
 
@@ -97,8 +97,9 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NG <= 2 ? 4 : 3) k_attn_f32(c
         return dense ? pos : col_bytes == 2 ? (int)col2[pos] : (int)col4[pos];
     };
     int idx = key(lane & 15);
-#pragma unroll 1
-    for (int base = 0; base < n; base += 16) {
+    // 16 keys from the row's position base on, fewer at the end of a row (FULL false)
+    auto step = [&](auto full, int base) {
+        constexpr bool FULL = decltype(full)::value;
         const int cnt = n - base;  // keys left
         const int next = key(base + 16 + (lane & 15));
         // scores of keys 4 r + kg at this lane's head
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NG <= 2 ? 4 : 3) k_attn_f32(c
                     sh[r][0] += __shfl_xor_sync(0xFFFFFFFFu, sh[r][0], lanes);
                     lanes >>= 1;
                 }
-                s[r] = 4 * r + kg < cnt ? sh[r][0] * a.scale_log2 : -INFINITY;
+                s[r] = FULL || 4 * r + kg < cnt ? sh[r][0] * a.scale_log2 : -INFINITY;
             }
         }
 
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NG <= 2 ? 4 : 3) k_attn_f32(c
             }
         }
 
-        // values, four keys per step (slots past the row have p = 0)
+        // values, four keys at a time
         uint64_t vb[2][4][DL / 2];
         auto load_v = [&](int r, uint64_t(&dst)[4][DL / 2]) {
 #pragma unroll
@@ -207,8 +208,16 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NG <= 2 ? 4 : 3) k_attn_f32(c
         load_v(0, vb[0]);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            if (4 * r >= cnt) break;
-            if (r + 1 < 4 && 4 * (r + 1) < cnt) load_v(r + 1, vb[(r + 1) & 1]);
+            if (!FULL && 4 * r >= cnt) break;
+            if (r + 1 < 4 && (FULL || 4 * (r + 1) < cnt)) load_v(r + 1, vb[(r + 1) & 1]);
+            if (!FULL) {
+                // slots past the row hold the row's own values, which may be infinite: p = 0 is not enough
+#pragma unroll
+                for (int x = 1; x < 4; ++x)
+#pragma unroll
+                    for (int e = 0; e < DL / 2; ++e)
+                        if (4 * r + x >= cnt) vb[r & 1][x][e] = 0ull;
+            }
 #pragma unroll
             for (int x = 0; x < 4; ++x)
 #pragma unroll
@@ -219,6 +228,18 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NG <= 2 ? 4 : 3) k_attn_f32(c
                 }
         }
         idx = next;
+    };
+    // The full steps have a body of their own: setting aside the slots past the row in a common one takes the larger
+    // groups 5% (12 / 2 heads, N = 6007: 274 us without, 288-292 with, 249 with two bodies); the
+    // smaller ones are 1 us faster with one (one head, N = 2048: 29.4 against 31-32 us).
+    int base = 0;
+    if constexpr (NG > 2) {
+#pragma unroll 1
+        for (; base + 16 <= n; base += 16) step(std::true_type{}, base);
+        if (base < n) step(std::false_type{}, base);
+    } else {
+#pragma unroll 1
+        for (; base < n; base += 16) step(std::false_type{}, base);
     }
 
     // row sums over the key groups, normalise, store

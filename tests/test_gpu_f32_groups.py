@@ -22,3 +22,20 @@ def test_f32_groups(Hq, Hkv, D, N, mode, d):
     # the same sums rounded to bf16: half an ulp, and one flip of the rounding by the fp32 error
     half, _ = run_gpu(q, k, v, mode, d, [1, 2], 3, 1e4, 64, out_dtype=torch.bfloat16)
     assert (np.abs(to_np(half) - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5).all()
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(2, 2, 64), (4, 2, 128), (12, 2, 128)])
+def test_f32_infinite_values_stay_infinite(Hq, Hkv, D):
+    """A row whose own value is infinite comes out infinite, whatever the row's length leaves of the kernel's
+    last step; rows and channels without one come out as they are."""
+    N = 70
+    (q, k, v), _ = make_inputs(N, Hq, Hkv, D, dtype=torch.float32, seed=D)
+    ref, _ = run_gpu(q, k, v, 2, 1.0, [1], 0, 1e4, 64)
+    keys = [13, 34, 36, 69]
+    for c, j in enumerate(keys):
+        v[j, :, c] = float("inf") if c % 2 == 0 else -float("inf")
+    out, lse = run_gpu(q, k, v, 2, 1.0, [1], 0, 1e4, 64)
+    for c, j in enumerate(keys):
+        assert torch.equal(out[:j, :, c], ref[:j, :, c])
+        assert (out[j:, :, c] == v[j, 0, c]).all()
+    assert torch.equal(out[:, :, len(keys):], ref[:, :, len(keys):]) and torch.isfinite(lse).all()
