@@ -182,7 +182,10 @@ ris_status ris_rope_apply(void *x, int32_t dtype, int64_t N, int32_t heads, int3
  * with one softmax over the whole key set M_i of the master mask (all seeds OR-merged), q~ and
  * k~ rotated by `rope` (NULL or kind NONE: q and k are used as given). Builds the mask, runs
  * the attention and frees the mask, all on `stream`; blocks once while the mask is sized, unless the
- * key lists of every causal pair would fit in 64 MiB (about N = 8190).
+ * key lists of every causal pair would fit in 64 MiB (about N = 8190). Such a call does not know the
+ * mask's pair count and chooses its design (see ris_attention_design) from the expected one: near the
+ * line between two designs it may take the other than ris_attention_masked on the built mask, with
+ * outputs that differ in their last bits.
  * dtype: q, k, v element type; out_dtype: out element type (F32 or BF16). lse: optional
  * [heads][N] fp32 natural-log sum of exp of the scaled scores (NULL to skip).
  * head_dim in {64, 128}; heads a multiple of kv_heads; heads/kv_heads <= 8, or any group size

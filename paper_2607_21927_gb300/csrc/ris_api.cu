@@ -467,9 +467,15 @@ ris_status ris_rope_freqs(const ris_rope_cfg *rope, int64_t N, int32_t head_dim,
 namespace {
 
 // Expected pairs of all masks of a call: the forced keys, and the others with the probability that one
-// of a mask's seeds draws them.
-double expected_pairs(const ris_mask_s *m, const ris_mask_opts &o)
+// of a mask's seeds draws them (a seed given twice draws the same keys).
+double expected_pairs(const ris_mask_s *m, const ris_mask_opts &o, const uint32_t *seeds)
 {
+    double draws_of_a_key = 1.0;
+    if (!m->per_seed) {
+        std::vector<uint32_t> s(seeds, seeds + m->n_seeds);
+        std::sort(s.begin(), s.end());
+        draws_of_a_key = (double)(std::unique(s.begin(), s.end()) - s.begin());
+    }
     const double n = (double)m->N, causal = n * (n + 1.0) / 2.0;
     const ris_params &p = m->params;
     const double hit = o.sampler == 1 ? 1.0 - std::pow(1.0 - 1.0 / n, (double)p.draws) : (double)p.thr / 4294967296.0;
@@ -477,7 +483,7 @@ double expected_pairs(const ris_mask_s *m, const ris_mask_opts &o)
     const double anchors = std::min((double)o.n_anchor, n);
     const double forced = std::min(causal, (double)suffix_pairs_of(m->N, block, o.local_window) +
                                                anchors * std::max(0.0, n - std::max<double>(o.local_window, (double)block)));
-    return m->n_masks * (forced + (causal - forced) * (1.0 - std::pow(1.0 - hit, m->per_seed ? 1.0 : (double)m->n_seeds)));
+    return m->n_masks * (forced + (causal - forced) * (1.0 - std::pow(1.0 - hit, draws_of_a_key)));
 }
 
 // Key lists of up to this many bytes, if every causal pair were kept, are allocated at that size by the
@@ -577,7 +583,7 @@ ris_status build_mask(int64_t N, int32_t kv_heads, int32_t mode, double density,
 
     int64_t room = n_masks * (N * (N + 1) / 2);  // at most: every causal pair
     if (!sized && room <= kUnsizedBytes / mk->col_bytes) {
-        mk->n_pairs = (int64_t)(expected_pairs(mk, o) + 0.5);
+        mk->n_pairs = (int64_t)(expected_pairs(mk, o, seeds) + 0.5);
     } else {
         RIS_CUDA(cudaMemcpyAsync(&room, mk->row_ptr + n_rows, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         RIS_CUDA(cudaStreamSynchronize(s));

@@ -24,3 +24,14 @@ def test_one_call_equals_prebuilt_mask(N, mode, d, S, W, A, sampler, dtype):
         with ris.ris_mask_generate(N, 2, mode, d, seeds, opts, per_seed=per_seed) as m:
             ref, ref_lse = ris.ris_attention_masked(m, q, k, v, rope, out_dtype=torch.float32, return_lse=True)
         assert torch.equal(out, ref) and torch.equal(lse, ref_lse)
+
+
+@pytest.mark.parametrize("mode,d,A", [(0, 0.01, 0), (1, 0.01, 4)], ids=["stochastic", "blocks"])
+def test_seeds_given_twice_count_once(mode, d, A):
+    """Twenty times the same seed keep what one keeps, and the one call takes the design of that mask."""
+    q, k, v = make_inputs(3001, 8, 2, 64, seed=9)[0]
+    seeds, opts, rope = [7] * 20, ris.mask_opts(1, A), ris.rope_cfg(3, 1e6, 1024)
+    out = ris.ris_sparse_attention_fwd(q, k, v, mode, d, seeds, rope=rope, opts=opts, out_dtype=torch.float32)
+    with ris.ris_mask_generate(3001, 2, mode, d, seeds, opts) as m:
+        assert ris.ris_attention_design(m, torch.bfloat16, 64) == 0
+        assert torch.equal(out, ris.ris_attention_masked(m, q, k, v, rope, out_dtype=torch.float32))
