@@ -233,16 +233,13 @@ int64_t range_sum(int64_t a, int64_t b) { return b > a ? (a + b - 1) * (b - a) /
 int64_t suffix_pairs_of(int64_t N, int64_t block, int64_t W)
 {
     if (W < 1) W = 1;
-    if (block <= 0) return N <= W ? range_sum(1, N + 1) : range_sum(1, W + 1) + (N - W) * W;
-    int64_t total = 0;
-    for (int64_t b0 = 0; b0 < N; b0 += block) {
-        const int64_t b1 = std::min(N, b0 + block);
-        total += range_sum(b0 + 1, std::min(b1, W) + 1);                  // i < W: i + 1 keys
-        const int64_t s = std::max(b0, W);                                // i >= W:
-        total += std::max<int64_t>(0, std::min(b1, b0 + W) - s) * W;     //   i - b0 < W: W keys
-        total += range_sum(W + 1, b1 - b0 + 1);                           //   else i - b0 + 1 keys
-    }
-    return total;
+    const int64_t head = range_sum(1, std::min(N, W) + 1);
+    if (N <= W) return head;
+    if (block <= 0) return head + (N - W) * W;
+    // rows of a block at offsets 0 .. n - 1, all at or past W
+    auto rows = [&](int64_t n) { return std::min(n, W) * W + range_sum(W + 1, n + 1); };
+    const int64_t b0 = W / block * block, b1 = std::min(N, b0 + block);  // the block that holds row W
+    return head + rows(b1 - b0) - rows(W - b0) + (N - b1) / block * rows(block) + rows((N - b1) % block);
 }
 
 // Design of a layer call: 0 register gather, 2 masked dense tiles, 3 fp32
