@@ -239,7 +239,9 @@ ris_status ris_attention_masked_rows(ris_mask_t mask, int64_t row_begin, int64_t
  * rows in which each device holds only its own rows of q, k and v and all-gathers the layer's
  * K and V first (the paper's row independence, Methods, "Memory-Bounded Geometry Generation":
  * every device builds the same counter-based mask). Each row equals the same row of the
- * whole-layer call bit for bit. Masks built per seed are refused (RIS_ERR_UNSUPPORTED).
+ * whole-layer call bit for bit, except that with rotated bf16 inputs at head dim 128 the power-of-two
+ * scales of the score operands follow from the largest pair norm (elements c and c + 64) of the queries
+ * given: where the whole layer's is in another binade, last bits may differ. Masks built per seed are refused (RIS_ERR_UNSUPPORTED).
  * Errors: as ris_attention_masked_rows. */
 ris_status ris_attention_masked_local(ris_mask_t mask, int64_t row_begin, int64_t row_end, const void *q_rows,
                                       const void *k, const void *v, void *out_rows, int32_t heads, int32_t kv_heads,
@@ -290,7 +292,8 @@ ris_status ris_noalloc_scratch_info(void **device_address, int64_t *bytes);
 
 /* Kernel timer for measurement (off by default). While enabled, every attention kernel launch
  * (the fused QK^T -> softmax -> PV kernel of a layer, or a decode step's two kernels; not
- * RoPE or mask kernels) is bracketed by CUDA events recorded on the stream it is launched on. Enabling or disabling clears the record.
+ * RoPE or mask kernels) is bracketed by CUDA events recorded on the stream it is launched on. Enabling or
+ * disabling clears the record.
  * ris_kernel_timer_read blocks until the last recorded launch has finished, returns the summed
  * device milliseconds and the number of launches recorded since the last read, and clears
  * them. Intended for one thread at a time. Errors: RIS_ERR_INVALID (NULL outputs), RIS_ERR_CUDA. */
@@ -305,8 +308,8 @@ ris_status ris_kernel_timer_samples(double *total_ms, int64_t *launches, double 
  * 3 fp32 gather, 4 dense-suffix split; -1 for invalid arguments. bf16 calls use tiles when
  * the mask is dense or keeps at least 5.8% (head_dim 128) or 8.8% (head_dim 64) of the
  * causal pairs (up to 2.25 times that below 3072 tokens) in what a gather would fetch (and
- * always when heads/kv_heads > 8, which this call does not see). The dense-suffix split applies to masks (not per seed) with Structural
- * blocks of at least 256 tokens or a local window of at least 256 keys: every key of row i
+ * always when heads/kv_heads > 8, which this call does not see). The dense-suffix split applies to
+ * masks (not per seed) with Structural blocks of at least 256 tokens or a local window of at least 256 keys: every key of row i
  * from the earlier of its block start and its window start up to i is kept (Methods,
  * "Sampling Modes": in-block pairs are cliques; the window is forced), so a first launch
  * attends every row to that suffix on the tiles and the register gather continues that

@@ -46,40 +46,33 @@
 // undone in the epilogue.
 //
 // What bounds it: a tile takes 24 products of 128 x 128 x 16 slots (8 fp16 score products, 2 x 4
-// e4m3 corrections at twice the rate, 8 fp16 value products), 1,536 cycles of the tensor pipe.
-// Measured per tile with clock64() stamps in the longest CTA of a 32k dense / 64k 10% layer:
-//   2,485 / 2,650 cycles  P over the score columns, one lane issuing inside a branch, two threads
-//                         per row in lockstep: each product cost the issuing lane about 60 cycles of
-//                         operand moves, as long as the product, plus its waits;
-//   2,055 / 2,400         operands warp-uniform and issued by an elected lane: the softmax, its two
-//                         threads per row meeting in every tile, set the pace;
-//   1,860 / 2,040         the two groups on alternate tiles, half a period apart; a separate warp
-//                         for the value products then made it 2,030 / 2,170: 96 KB of keys and
-//                         values per tile and SM (17 TB/s at this pace) came in too late;
-//   1,720 / 1,985         tiles shared by two SMs;
-//   1,620 / 1,950         P double-buffered: dense, the tensor pipe is 95% busy and the power limit
-//                         holds the clock at 1.58 GHz; with a bitmap the softmax (about 450 cycles of
-//                         masking per tile more) is as slow as the pipe. There the groups' warps of a
-//                         scheduler ran their exponentials against each other, and a warp in a
-//                         hundred rescaled O, while seven others waited: the reference maximum is now
-//                         handed over after the exponentials (it still moves at 2^8: at 2^14 the heaviest
-//                         weight of a row is less often exactly 1, and the log-sum-exp of a dense
-//                         32k layer is 5% further off);
-//                         (the waits of the softmax on what the products did are relaxed: acquiring at
-//                         cluster scope there, at 8k and 64k, made a layer 1.2-1.5% slower);
-//   1,650 / 1,870         row sums that add fp16 as it is, -infinity by predicated moves, the next
-//                         tile's scores polled for ahead of their use. Then O is rescaled after the
-//                         exponentials and the hand-over instead of before: N = 8192 230 -> 226 us.
-// A CTA's start and end, 16,000 cycles with the query rows loaded and the output rows stored 16 bytes
-// per lane and row, take 7,000 with the query tile loaded by TMA and the output through
-// shared memory; the first loads ahead of the TMEM allocation and the cluster barrier then took N =
-// 8192 from 224 to 221 us.
-// Layer calls, before -> now: N = 8192 306 -> 222 us, 32k dense 3.75 -> 2.90 ms, 64k
-// 14.0 -> 11.1 ms.
-// Not kept: the bitmap applied to P as packed masks, with the maximum taken over all keys and again
-// over the kept ones only where it could move (fewer instructions, but in the exponentials' chain
-// from group to group: N = 8192 226 -> 244 us), more polls between two reads of the error word in a
-// wait (3% slower at N = 8192), a suspend-time hint on the polls (no change).
+// e4m3 corrections at twice the rate, 8 fp16 value products), 1,536 cycles of the tensor pipe. A
+// dense 32k layer takes about 1,650 cycles per tile: the pipe is 95% busy and the power limit holds
+// the clock at 1.58 GHz. With a bitmap (64k, 10%) 1,870, where the softmax with about 450 cycles of masking is
+// as slow as the pipe. Layer calls: N = 8192 220-226 us, 32k dense 2.85 ms, 64k 11.0-11.4 ms.
+// Why it is laid out so (in brackets cycles per tile of the dense / the masked layer from clock64()
+// stamps, or a layer's time, the other way against this one):
+//   - products are issued with warp-uniform operands by an elected lane: inside a branch on the lane
+//     each costs the issuing lane about 60 cycles of operand moves, as long as the product itself
+//     (2,485 / 2,650, against 2,055 / 2,400);
+//   - two softmax groups on alternate tiles, half a period apart: with two threads per row on every
+//     tile their meeting set the pace (2,055 / 2,400, against 1,860 / 2,040);
+//   - key and value tiles shared by two SMs: 96 KB per tile and SM, 17 TB/s at this pace, come in too
+//     late (2,030 / 2,170, against 1,720 / 1,985);
+//   - P double-buffered, in columns of its own (1,720 / 1,985, against 1,620 / 1,950);
+//   - the reference maximum is handed over after the exponentials, and O rescaled after that: the groups' warps
+//     of a scheduler otherwise run their exponentials against each other, and a warp in a hundred
+//     that rescales O holds up seven others (N = 8192: 230, against 226 us);
+//   - the reference maximum moves at 2^8: at 2^14 the heaviest weight of a row is less often exactly 1, and
+//     the log-sum-exp of a dense 32k layer is 5% further off;
+//   - row sums that add fp16 as it is, -infinity by predicated moves, the next tile's scores polled for
+//     ahead of their use (masked 1,950, against 1,870; a dense layer is not held by the softmax). The
+//     bitmap applied to P as packed masks has fewer instructions, but they lie in the chain of
+//     exponentials from group to group (N = 8192: 244, against 226 us);
+//   - waits of the softmax warps on products are relaxed at cluster scope: acquiring there takes a masked
+//     layer 1.2-1.5% longer;
+//   - the query tile by TMA and the output through shared memory: with rows loaded and stored 16 bytes per
+//     lane a CTA's start and end take 16,000 cycles instead of 7,000.
 //
 // The suffix pass of the dense-suffix split (SUFFIX) runs the same pipeline over the key
 // tiles of each row's dense suffix only (its Structural block and / or local window: every key
@@ -137,9 +130,9 @@ constexpr uint32_t kTmemCols = 512;  // S (2 x 128) + O (128) + P (2 x 64)
 // 64-byte rows; each CTA works for itself there.
 //
 // Shared memory (bytes, from a 1024-aligned base): the K ring, the V ring, the query tile (hi part,
-// low part), then the barriers, the TMEM base and what the two threads of a row hand to each
-// other: the row's reference maximum after each tile, and at the end each thread's row sum and
-// the maximum it refers to.
+// low part), then the barriers, the TMEM base, the notes for the end and what the two softmax groups
+// hand to each other for a row: its reference maximum after each tile, and at the end each group's
+// row sum over its tiles and the maximum that sum refers to.
 template <int DT>
 struct Lay {
     static constexpr int CG = DT == 128 ? 2 : 1;
@@ -909,8 +902,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
         };
         // value product of a tile of ring stage ST: P (in TMEM, the buffer of the tile's parity), 128
-        // keys of fp16 values packed two per column, times V, 64 keys x 128 B rows per block: 16 keys = two 8-row atoms (SBO 1024); the
-        // second 64-column block of head dim is LBO = 16 KB away
+        // keys of fp16 values packed two per column, times V, 128 keys x 128 B rows per block: 16 keys = two
+        // 8-row atoms (SBO 1024); the second 64-column block of head dim is LBO = 16 KB away
         auto issue_o = [&](auto st_c, uint32_t acc) {
             constexpr int ST = decltype(st_c)::value;
             const uint32_t vd = desc_lo(sbase + L::OFF_V + ST * L::V_STAGE, L::V_BLK);
@@ -979,7 +972,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
         const float sc = a.scale_log2;
         const float v_absmax = *a.v_absmax;
-        if (lane == 0 && grp < n_kt) arrive_lead(L::B_S_GO + grp);  // the group's score buffer is free for its first tile
+        // the group's score buffer is free for its first tile
+        if (lane == 0 && grp < n_kt) arrive_lead(L::B_S_GO + grp);
         // kept keys of word e of tile j (keys 128 (kt0 + j) + 32 e .. +31): the bitmap's word, or
         // the range suffix_lo .. i (dense: 0 .. i)
         constexpr bool kRange = DENSE || SUFFIX;
@@ -1021,7 +1015,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool s_full = false;  // seen at the end of the last tile: a poll takes 200 cycles even if it succeeds
         for (int j = grp; j < n_kt; j += 2) {
             if (!kRange) mask_words(j + 4, nnw);
-            if (ok) ok = __all_sync(0xFFFFFFFFu, s_full || mbar_wait<CG, true>(sbase + BAR(L::B_S_FULL + j % NSK), (j / NSK) & 1, wl));
+            if (ok) {
+                const uint32_t bar = sbase + BAR(L::B_S_FULL + j % NSK);
+                ok = __all_sync(0xFFFFFFFFu, s_full || mbar_wait<CG, true>(bar, (j / NSK) & 1, wl));
+            }
             tc_fence_after();
             uint32_t su[2][64];
             tmem_issue64(T_S0 + grp * BN + lane_off, su[0]);
@@ -1063,8 +1060,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             const float mx =
                 fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * sc;
-            // The row's reference maximum moves on from tile to tile, handed to the other group. Lazy rescale: it moves, and O is rescaled, only when the row max
-            // grows by more than kLazyLog2. The TMEM loads / stores are warp-collective
+            // The row's reference maximum moves on from tile to tile, handed to the other group. Lazy
+            // rescale: it moves, and O is rescaled, only when the row max grows by more than
+            // kLazyLog2. The TMEM loads / stores are warp-collective
             // (.sync.aligned), so the whole warp runs them when any of its rows needs it; the
             // other rows multiply by 1.
             float m_prev = -INFINITY;
@@ -1076,7 +1074,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             const float m_ref = upd ? mx : m_prev;
             // the value product of tile t is done (t < 0: nothing to wait for)
             auto pv_done = [&](int t) -> bool {
-                return t < 0 || __all_sync(0xFFFFFFFFu, mbar_wait<CG, true>(sbase + BAR(L::B_PV_DONE + t % NSV), (t / NSV) & 1, wl));
+                const uint32_t bar = sbase + BAR(L::B_PV_DONE + t % NSV);
+                return t < 0 || __all_sync(0xFFFFFFFFu, mbar_wait<CG, true>(bar, (t / NSV) & 1, wl));
             };
             const bool scale_o = upd && m_prev != -INFINITY;
             const bool any_scale = __any_sync(0xFFFFFFFFu, scale_o);
@@ -1117,10 +1116,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) continue;
             tc_fence_after();
             if (any_scale) {
-                // O has settled once the value product of tile j - 1 is done (that of tile j - 2 first, above, so
-                // that the barrier is not polled a phase early); nothing adds to it before this warp's
-                // P is announced below, and the other group's warp of these rows scales it next only after that product.
-                // Here and not ahead of the exponentials, where the wait held up the other group as well.
+                // O has settled once the value product of tile j - 1 is done (that of tile j - 2 first,
+                // above, so that the barrier is not polled a phase early); nothing adds to it before
+                // this warp's P is announced below, and the other group's warp of these rows scales it next
+                // only after that product. Here and not ahead of the exponentials, where the wait held
+                // up the other group as well.
                 ok = pv_done(j - 1);
                 if (!ok) continue;
                 tc_fence_after();

@@ -67,8 +67,8 @@ struct RowDraws {
 // over seeds: it asks after `first_vote` seeds and then every kVoteSeeds.
 //
 // Philox4x32-10 as in philox4x32_10 above, with what the 10 rounds of a row's calls have in common
-// taken out of the loop over seeds (SEEDS a pass; 0: one seed in all, s0, without a loop or minima). Round 1 multiplies the group (word 0) and the stream (word 2),
-// neither of which depends on the seed; its results z, w depend on the group only (key word 1 is
+// taken out of the loop over seeds (unrolled by SEEDS; 0: one seed in all, s0, without a loop or
+// minima). Round 1 multiplies the group (word 0) and the stream (word 2), neither of which depends on the seed; its results z, w depend on the group only (key word 1 is
 // the head key) and x, y on the row and seed only. So the second product of round 2 depends on the
 // group only and the first on the seed only: per call 8 rounds of two products remain, 16 of 20.
 constexpr int kVoteSeeds = 4;
@@ -197,11 +197,11 @@ __device__ __forceinline__ int row_step(const MaskBitsArgs &a, const RowTask &t,
 //
 // Bound by the 32 x 32 -> 64-bit products (32 lanes per clock and SM, a quarter of the fp32 rate)
 // and, nearly as much, by the ALU pipe (an exclusive or per product, the minima, the key schedule).
-// SEEDS = 2: as many registers as the compiler wants (the key schedules stay in registers). Measured at N =
-// 16384 of 1% (one seed per pass and eight CTAs per SM / two per pass): 2 seeds 217 / 209 us, 3 297 / 283,
-// 8 693 / 641, 20 1644 / 1487. 70 seeds at N = 32768: 29.0 ms with every round in the loop over seeds and one thread
-// per word, 21.1 with rounds 1 and 2 taken out, 19.6 now (1.5 calls per clock and SM). SEEDS = 0, one seed: eight
-// CTAs per SM, a row's other work counts.
+// SEEDS = 2, two or more seeds: two a pass and as many registers as the compiler wants, which keeps the key schedules
+// in registers (N = 16384 of 1%, against one a pass and eight CTAs per SM: 2 seeds 209 / 217 us, 3 283 / 297, 8 641 /
+// 693, 20 1487 / 1644). 70 seeds at N = 32768 take 19.6 ms, 1.5 calls per clock and SM (21.1 one a pass, 29.0
+// with rounds 1 and 2 in the loop over seeds and a thread per word). SEEDS = 0, one seed: eight CTAs
+// per SM, as a row's other work counts.
 template <int SEEDS>
 __global__ void __launch_bounds__(kBitsThreads, SEEDS > 0 ? 1 : 8) k_mask_bits(const MaskBitsArgs a, int first_vote)
 {
@@ -227,9 +227,8 @@ __global__ void __launch_bounds__(kBitsThreads, SEEDS > 0 ? 1 : 8) k_mask_bits(c
 
 // One seed per mask and rows enough for four of them per CTA (the caller sees to both): the steps of
 // the four rows one after the other, dealt to the warps in turn. With one call per four keys a CTA's
-// start, its last step and its end are a good part of a short row: ten one-seed masks of N = 8192 take 345 us
-// against 360 with one row per CTA (367 with the loop over seeds and its minima), one of N = 16384 121-127
-// against 130 (138).
+// start, its last step and its end are a good part of a short row: ten one-seed masks of N = 8192 take
+// 345 us (360 with a row per CTA, 367 with the loop over seeds besides), one of N = 16384 121-127 (130, 138).
 constexpr int kOneSeedRows = 4;
 __global__ void __launch_bounds__(kBitsThreads, 6) k_mask_bits_one(const MaskBitsArgs a)
 {
