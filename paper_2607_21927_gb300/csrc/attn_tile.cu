@@ -49,7 +49,7 @@
 // e4m3 corrections at twice the rate, 8 fp16 value products), 1,536 cycles of the tensor pipe. A
 // dense 32k layer takes about 1,650 cycles per tile: the pipe is 95% busy and the power limit holds
 // the clock at 1.58 GHz. With a bitmap (64k, 10%) 1,870, where the softmax with about 450 cycles of masking is
-// as slow as the pipe. Layer calls: N = 8192 220-226 us, 32k dense 2.85 ms, 64k 11.0-11.4 ms.
+// as slow as the pipe. Layer calls: N = 8192 226 us, 32k dense 2.9 ms, 64k 11.4 ms.
 // Why it is laid out so (in brackets cycles per tile of the dense / the masked layer from clock64()
 // stamps, or a layer's time, the other way against this one):
 //   - products are issued with warp-uniform operands by an elected lane: inside a branch on the lane
@@ -719,6 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int kt0 = SUFFIX ? (int)(dense_suffix_start(a, (int64_t)max(qt_lo, qt_first) * BM) / BN) : 0;
     const int n_kt = (int)(last_row / BN) + 1 - kt0;
 
+    constexpr auto BAR = [](int i) { return (uint32_t)(L::OFF_BARS + 8 * i); };
     const bool first_loads = a.debug_no_loads == 0 && (sbase & 1023u) == 0u;
     if (warp == kTmaWarp) {
         static_assert(L::NBAR <= 32, "a lane per barrier");
@@ -733,30 +734,32 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (lane < (int)(sizeof(ClosingNotes) / 4)) reinterpret_cast<volatile uint32_t *>(smem + L::OFF_END)[lane] = 0u;
         __syncwarp();
-    }
-    // The barriers of both CTAs are initialised once this cluster barrier is passed. (That the other CTA's
-    // tensor memory is allocated before a product writes to it follows from its softmax warps'
-    // first arrivals.)
-    if constexpr (CG == 2) cluster_arrive();
-    if (warp == kScoreWarp) tmem_alloc<CG>(smem_u32(&tmem_base_sh));  // by one full warp (of each CTA)
-    if constexpr (CG == 2) cluster_wait();
-    const uint32_t lead = CG == 2 ? cluster_addr(sbase, 0) : sbase;  // the issuing CTA's shared memory
-    constexpr auto BAR = [](int i) { return (uint32_t)(L::OFF_BARS + 8 * i); };
-    // the query tile and the first keys at once, under the rest of the start-up (about 2,000 cycles, the
-    // TMEM allocation most of them)
-    if (warp == kTmaWarp && lane == 0 && first_loads) {
-        const uint32_t bq = lead + BAR(L::B_Q_FULL), bk = lead + BAR(L::B_K_FULL);
-        const int key = kt0 * BN + L::KROWS * rank;
-        mbar_arrive_expect_tx<CG>(bq, (SPLIT ? 2 : 1) * L::Q_ARR);
-        mbar_arrive_expect_tx<CG>(bk, (SPLIT ? 2 : 1) * L::K_ARR);
-        for (int blk = 0; blk < NB; ++blk) {
-            const int row = (int)(q0 - a.q_first);
-            tma_load_3d<CG>(sbase + L::OFF_Q + blk * L::Q_BLK, &maps.qh, 64 * blk, h, row, bq);
-            if (SPLIT) tma_load_3d<CG>(sbase + L::OFF_Q + L::Q_ARR + blk * L::Q_BLK, &maps.ql, 64 * blk, h, row, bq);
-            tma_load_3d<CG>(sbase + L::OFF_K + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
-            if (SPLIT) tma_load_3d<CG>(sbase + L::OFF_K + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
+        // The barriers of both CTAs are initialised once this cluster barrier is passed. (That the other CTA's
+        // tensor memory is allocated before a product writes to it follows from its softmax warps'
+        // first arrivals.)
+        if constexpr (CG == 2) cluster_sync();
+        // the query tile and the first keys at once, under the rest of the start-up (about 2,000 cycles, the
+        // TMEM allocation most of them). In this warp's branch: in the code of all warps the compiler spills
+        // around it, N = 8192 230 instead of 226 us.
+        if (lane == 0 && first_loads) {
+            const uint32_t lead = CG == 2 ? cluster_addr(sbase, 0) : sbase;
+            const uint32_t bq = lead + BAR(L::B_Q_FULL), bk = lead + BAR(L::B_K_FULL);
+            const int key = kt0 * BN + L::KROWS * rank, row = (int)(q0 - a.q_first);
+            mbar_arrive_expect_tx<CG>(bq, (SPLIT ? 2 : 1) * L::Q_ARR);
+            mbar_arrive_expect_tx<CG>(bk, (SPLIT ? 2 : 1) * L::K_ARR);
+            for (int blk = 0; blk < NB; ++blk) {
+                tma_load_3d<CG>(sbase + L::OFF_Q + blk * L::Q_BLK, &maps.qh, 64 * blk, h, row, bq);
+                if (SPLIT) tma_load_3d<CG>(sbase + L::OFF_Q + L::Q_ARR + blk * L::Q_BLK, &maps.ql, 64 * blk, h, row, bq);
+                tma_load_3d<CG>(sbase + L::OFF_K + blk * L::K_BLK, &maps.kh, 64 * blk, g, key, bk);
+                if (SPLIT) tma_load_3d<CG>(sbase + L::OFF_K + L::K_ARR + blk * L::K_BLK, &maps.kl, 64 * blk, g, key, bk);
+            }
         }
+    } else {
+        if constexpr (CG == 2) cluster_arrive();
+        if (warp == kScoreWarp) tmem_alloc<CG>(smem_u32(&tmem_base_sh));  // by one full warp (of each CTA)
+        if constexpr (CG == 2) cluster_wait();
     }
+    const uint32_t lead = CG == 2 ? cluster_addr(sbase, 0) : sbase;  // the issuing CTA's shared memory
     __syncwarp();
     tc_fence_before();
     __syncthreads();

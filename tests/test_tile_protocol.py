@@ -20,7 +20,8 @@ def test_commits_are_waited_for_in_each_cta():
     for target in targets:
         bar = re.fullmatch(r"sbase \+ BAR\(L::(B_\w+) \+ ST\)", target)
         assert bar, f"commit to a barrier of its own: {target}"
-        assert re.search(rf"mbar_wait<CG[^>]*>\(sbase \+ BAR\(L::{bar[1]} \+ ", SOFTMAX), bar[1]
+        # (softmax warps arrive on barriers only through arrive_lead: an address taken here is waited on)
+        assert re.search(rf"(mbar_(wait|test)<CG[^>]*>\(|uint32_t bar = )sbase \+ BAR\(L::{bar[1]} \+ ", SOFTMAX), bar[1]
         assert f"mbar_wait_own<CG>(sbase + BAR(L::{bar[1]} + " in CLOSING, bar[1]
     # the second wait of the closing part ends before either CTA leaves
     assert CLOSING.index("mbar_wait_own") < CLOSING.rindex("cluster_sync()") < CLOSING.index("tmem_dealloc<CG>(tmem)")
@@ -57,7 +58,6 @@ def test_copies_complete_on_the_issuing_ctas_barriers():
     assert any("cta_group::2" in s for s in loads)
     assert not re.search(r"tma_load_3d\(", KERNEL)  # the form is chosen by the number of CTAs
     for bar in ("bq", "bk", "bv"):
-        assert re.search(rf"\b{bar} = lead \+ BAR\(", KERNEL), bar
-        assert not re.search(rf"\b{bar} = sbase ", KERNEL), bar
+        assert re.findall(rf"\b{bar} = (\w+)", KERNEL).count("lead") == len(re.findall(rf"\b{bar} = ", KERNEL)) > 0, bar
     relay = KERNEL[KERNEL.index("=== relay"):KERNEL.index("=== product issuers")]
     assert "arrive_lead" not in relay and relay.count("mbar_arrive(sbase + BAR(") == 2
