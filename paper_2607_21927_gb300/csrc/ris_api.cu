@@ -469,9 +469,10 @@ double expected_pairs(const ris_mask_s *m, const ris_mask_opts &o, const uint32_
 {
     double draws_of_a_key = 1.0;
     if (!m->per_seed) {
-        std::vector<uint32_t> s(seeds, seeds + m->n_seeds);
-        std::sort(s.begin(), s.end());
-        draws_of_a_key = (double)(std::unique(s.begin(), s.end()) - s.begin());
+        uint32_t s[kMaxSeeds];
+        std::copy(seeds, seeds + m->n_seeds, s);
+        std::sort(s, s + m->n_seeds);
+        draws_of_a_key = (double)(std::unique(s, s + m->n_seeds) - s);
     }
     const double n = (double)m->N, causal = n * (n + 1.0) / 2.0;
     const ris_params &p = m->params;
